@@ -20,8 +20,6 @@ NVCC_FLAGS = [
     # IEEE arithmetic everywhere: no FMA contraction, exact division and root, subnormals kept
     "--fmad=false", "--prec-div=true", "--prec-sqrt=true", "--ftz=false",
     "-Xcompiler", "-fPIC", "-shared",
-    # the kernels of a file are compiled side by side: 110 s -> 45 s on 8 cores
-    "--split-compile=0", "--threads", "2",
 ]
 
 
