@@ -176,8 +176,9 @@ def algorithmic_bytes(kernel: str, w, placement: str, D: int, gbits: int, xbits:
     """Bytes one launch of `kernel` must move at its interface (fp32 state it has
     to read and write, packed codes), for all n workers.  The worker side is capacity
     aware: (worker, segment) pairs that fit on chip go through the fused kernel and are
-    counted once (one pass); larger ones take the two streaming launches and are counted
-    twice (the max-abs scale needs the whole pair before any of it can be quantized)."""
+    counted once (one pass); larger ones take the two streaming launches: a sweep that settles
+    most of them, or two passes (the max-abs scale needs the whole pair before any of it can be
+    quantized)."""
     n = w.n
     server_moments = placement == "server"
     # with the l2 term a worker also reads the weights it holds: the packed broadcast, or x
@@ -188,6 +189,11 @@ def algorithmic_bytes(kernel: str, w, placement: str, D: int, gbits: int, xbits:
         return one_pass * ((12.0 if server_moments else 28.0) + held + gbits / 8.0)
     # the split launches cover everything, or, beside the fused kernel, the two-pass pairs only
     split_units = pass_model[1] if pass_model and pass_model[0] > 0 else n * D
+    # ternary and five-level codes, moments on the server: the sweep settles every row it can in one
+    # pass, and what its second kernel reads again (rows whose codes are not all level 0, which
+    # depends on the data) is not counted
+    if server_moments and w.kg in (0, 1) and kernel in ("absmax", "quantize"):
+        return (12.0 + held + gbits / 8.0) * split_units if kernel == "absmax" else 0.0
     if kernel == "absmax":      # phase 1: read g, e (worker moments: + read m, v, write m, v, u)
         per = (8.0 if server_moments else 28.0) + held
         return per * split_units

@@ -73,7 +73,7 @@ struct Geometry {
   std::vector<RTile> rtiles;
   std::vector<Tile> btiles;
   long long resident_elems = 0;      // padded elements of the resident segments (one vector)
-  size_t off_rtiles = 0, off_btiles = 0, off_words = 0;
+  size_t off_rtiles = 0, off_btiles = 0, off_words = 0, off_deferred = 0;
   size_t words_bytes = 0;            // room for the per-(pair, CTA) words of the on-chip worker kernel
 };
 
@@ -112,6 +112,17 @@ int validate_config(const qadam_config* c) {
       !(c->eps > 0.0f) || !std::isfinite(c->eps) || !std::isfinite(c->lr))
     return QADAM_ERR_HYPER;
   return QADAM_OK;
+}
+
+// Pairs that do not fit on chip: one sweep plus the rows it leaves, or two full passes.  The
+// sweep finishes a row whose codes are all level 0 without knowing the scale.  That needs u
+// unquantized (moments on the server: with them on the workers phase 1 writes u whatever the
+// codes turn out to be, and they are dense), and it pays where level 0 is wide: half or a
+// quarter of the scale.  Finer grids leave hardly a row (uniform, k_g = 3, Gaussian gradients,
+// 5 x 10^7 elements: 252 us against 217 in two passes), and the stochastic operator's level 0
+// depends on the coin.
+bool sweeps(const qadam_config* c, GMode gmode) {
+  return c->placement == QADAM_PLACE_SERVER && (gmode == G_TERNARY || gmode == G_FIVE);
 }
 
 int build_geometry(const qadam_config* c, Geometry* g) {
@@ -183,6 +194,10 @@ int build_geometry(const qadam_config* c, Geometry* g) {
     g->words_bytes = want <= kWordBudget ? want : 0;
     wo += (size_t)round_up64((int64_t)g->words_bytes, 256);
   }
+  // flags of the rows the sweep leaves to the second kernel (1 / 8192 of the size of e)
+  g->off_deferred = wo;
+  if (sweeps(c, g->gmode))
+    wo += 256 + (size_t)round_up64((int64_t)c->n * (int64_t)g->tiles.size() * kTileChunks, 256);   // a count first
   g->workspace_bytes = wo + 256;
   return QADAM_OK;
 }
@@ -219,6 +234,7 @@ struct qadam_ctx {
   size_t res_smem = 0;
   RTile* d_rtiles = nullptr;
   Tile* d_btiles = nullptr;
+  unsigned char* d_deferred = nullptr;
   unsigned long long* d_words = nullptr;   // nullptr: one counter per pair instead
   // qadam_step_host: the copy of worker i + 1 runs on a stream of its own while worker i is compressed
   cudaStream_t copy_stream = nullptr;
@@ -244,9 +260,15 @@ int resident_grid(K kernel, size_t smem, int sm_count) {
 using WorkerKernel = void (*)(const WorkerParams);
 using ServerKernel = void (*)(const ServerParams);
 
+// The first of the two streaming launches: max-abs, or the sweep that settles the rows it can.
 WorkerKernel pick_absmax(const qadam_ctx* c) {
   const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
-  if (c->lambda != 0.0f) return w ? worker_absmax_kernel<true, true> : worker_absmax_kernel<false, true>;
+  const bool l2 = c->lambda != 0.0f;
+  if (sweeps(&c->cfg, c->geo.gmode)) {
+    if (c->geo.gmode == G_TERNARY) return l2 ? worker_sweep_kernel<2, true> : worker_sweep_kernel<2, false>;
+    return l2 ? worker_sweep_kernel<3, true> : worker_sweep_kernel<3, false>;
+  }
+  if (l2) return w ? worker_absmax_kernel<true, true> : worker_absmax_kernel<false, true>;
   return w ? worker_absmax_kernel<true> : worker_absmax_kernel<false>;
 }
 
@@ -256,24 +278,28 @@ WorkerKernel pick_identity(const qadam_ctx* c) {
   return w ? worker_identity_kernel<true> : worker_identity_kernel<false>;
 }
 
+// The second: quantize everything, or the rows the sweep left.
+template <int MODE>
+WorkerKernel pick_quantize_mode(bool worker_moments, bool l2) {
+  if (worker_moments) return worker_quantize_kernel<true, MODE>;
+  // moments on the server: phase 2 forms u = g + e again, l2 term included
+  return l2 ? worker_quantize_kernel<false, MODE, true> : worker_quantize_kernel<false, MODE>;
+}
+template <int MODE>
+WorkerKernel pick_deferred_mode(bool worker_moments, bool l2) {
+  if (worker_moments) return worker_quantize_kernel<true, MODE>;
+  return l2 ? worker_deferred_kernel<MODE, true> : worker_deferred_kernel<MODE, false>;
+}
+
 WorkerKernel pick_quantize(const qadam_ctx* c) {
   const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
-  if (!w && c->lambda != 0.0f) {
-    // moments on the server: phase 2 forms u = g + e again, l2 term included
-    switch (c->geo.gmode) {
-      case G_STOCHASTIC: return worker_quantize_kernel<false, G_STOCHASTIC, true>;
-      case G_TERNARY: return worker_quantize_kernel<false, G_TERNARY, true>;
-      case G_FIVE:    return worker_quantize_kernel<false, G_FIVE, true>;
-      case G_POW2:    return worker_quantize_kernel<false, G_POW2, true>;
-      default:        return worker_quantize_kernel<false, G_UNIFORM, true>;
-    }
-  }
+  const bool l2 = c->lambda != 0.0f;
   switch (c->geo.gmode) {
-    case G_STOCHASTIC: return w ? worker_quantize_kernel<true, G_STOCHASTIC> : worker_quantize_kernel<false, G_STOCHASTIC>;
-    case G_TERNARY: return w ? worker_quantize_kernel<true, G_TERNARY> : worker_quantize_kernel<false, G_TERNARY>;
-    case G_FIVE:    return w ? worker_quantize_kernel<true, G_FIVE>    : worker_quantize_kernel<false, G_FIVE>;
-    case G_POW2:    return w ? worker_quantize_kernel<true, G_POW2>    : worker_quantize_kernel<false, G_POW2>;
-    default:        return w ? worker_quantize_kernel<true, G_UNIFORM> : worker_quantize_kernel<false, G_UNIFORM>;
+    case G_STOCHASTIC: return pick_quantize_mode<G_STOCHASTIC>(w, l2);
+    case G_TERNARY: return pick_deferred_mode<G_TERNARY>(w, l2);
+    case G_FIVE:    return pick_deferred_mode<G_FIVE>(w, l2);
+    case G_POW2:    return pick_quantize_mode<G_POW2>(w, l2);
+    default:        return pick_quantize_mode<G_UNIFORM>(w, l2);
   }
 }
 
@@ -488,6 +514,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     c->d_done = reinterpret_cast<unsigned*>(ws + c->geo.off_done);
     c->d_rtiles = reinterpret_cast<RTile*>(ws + c->geo.off_rtiles);
     c->d_btiles = reinterpret_cast<Tile*>(ws + c->geo.off_btiles);
+    c->d_deferred = ws + c->geo.off_deferred;
     c->d_words = c->geo.words_bytes ? reinterpret_cast<unsigned long long*>(ws + c->geo.off_words) : nullptr;
   }
 
@@ -655,13 +682,19 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
   p.seed_lo = (unsigned)c->cfg.seed;
   p.seed_hi = (unsigned)(c->cfg.seed >> 32);
   p.step = (unsigned)step;
+  p.deferred = c->d_deferred + 256;
+  p.deferred_rows = reinterpret_cast<unsigned*>(c->d_deferred);
 
-  // the two streaming launches over a tile table: max-abs, then quantize
+  // the two streaming launches over a tile table: max-abs, then quantize (or the sweep, then the
+  // rows it left)
   auto streaming = [&](const Tile* tiles, int tiles_per_worker) -> int {
     WorkerParams q = p;
     q.tiles = tiles;
     q.tiles_per_worker = tiles_per_worker;
     q.total_tiles = (long long)worker_count * tiles_per_worker;
+    if (sweeps(&c->cfg, c->geo.gmode) &&
+        !cuda_ok(cudaMemsetAsync(q.deferred_rows, 0, sizeof(unsigned), c->stream)))
+      return QADAM_ERR_CUDA;
     int grid = (int)std::min<int64_t>(c->grid_absmax, q.total_tiles);
     {
       LaunchTimer lt(c, QADAM_K_ABSMAX);

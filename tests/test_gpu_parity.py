@@ -339,6 +339,43 @@ def test_streaming_launches_only(placement):
     p.close()
 
 
+@pytest.mark.parametrize("kg,grid", [(0, 0), (1, 0), (2, 0), (3, 1)])
+@pytest.mark.parametrize("l2", [0.0, 5e-4])
+def test_streaming_sweep_settles_rows_before_the_scale_is_known(kg, grid, l2):
+    # Pairs too large for the chip (here: every pair, by option) are swept once; rows that a lower
+    # bound of the scale shows to be all level 0 are finished there, the others by a second kernel.
+    # Lengths around the rows of 128, chunks of 512 and tiles of 4096 elements; the maximum at the
+    # front, at the end and in the middle; coordinates exactly on the lowest midpoint and next to
+    # it; zeros of either sign, a segment of zeros, one of subnormal magnitudes.
+    import paper_2004_14180_b200 as qb
+    seg = [100, 512, 513, 1025, 4096, 4097, 3 * 4096 + 640, 150_000, 2048, 1024]
+    off = np.concatenate([[0], np.cumsum(seg)])
+    rng = np.random.default_rng(17 + kg)
+    d, n = sum(seg), 3
+    mid = np.float32(2.0 ** -(kg + 1))
+    x1 = (rng.standard_normal(d) * 0.2).astype(np.float32)
+    p = Pair(seg, n, kg, 0, S_MODE, x1=x1, grid_g=grid,
+             options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    if l2:
+        p.set_regularization(l2)
+    for t in range(3):
+        g = (rng.standard_normal((n, d)) * 1e-3).astype(np.float32)
+        big = np.float32(0.75 + t)
+        for w in range(n):
+            for s in range(len(seg)):
+                a, b = off[s], off[s + 1]
+                at = (a, b - 1, (a + b) // 2)[(w + s + t) % 3]
+                g[w, at] = big
+                if b - a > 600:
+                    at = a + 130 + 128 * ((w + t) % 3)
+                    g[w, at:at + 4] = [big * mid, -big * mid, np.nextafter(big * mid, np.float32(9)), -0.0]
+        g[:, off[8]:off[9]] = np.where(rng.random((n, seg[8])) < 0.5, np.float32(0.0), np.float32(-0.0))
+        g[:, off[9]:off[10]] = (rng.integers(-7, 8, (n, seg[9])) * 1e-45).astype(np.float32)
+        p.step(g, split_workers=t == 1)
+        p.compare_state()
+    p.close()
+
+
 # ---------------------------------------------------------------- l2 term and step-dependent rates
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
