@@ -232,6 +232,8 @@ struct qadam_ctx {
   int grid_resident = 0;
   int res_slots = 0, res_estages = 0;
   size_t res_smem = 0;
+  int res_slots_l2 = 0;          // with the l2 term: fewer slots, the stages carry the held weights too
+  size_t res_smem_l2 = 0;
   RTile* d_rtiles = nullptr;
   Tile* d_btiles = nullptr;
   unsigned char* d_deferred = nullptr;
@@ -592,8 +594,12 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     if (eligible) {
       // the CTA's shared memory: a ring of slots for u and a few stages for e (227 KB: 14 in all)
       const int estages = 2;                  // measured: 12 slots + 2 stages beat 11 + 3 and 10 + 4
-      const int slots = std::min(((int)max_smem - kRHeadBytes - estages * resident_stage_bytes(wm)) / kRSlotBytes,
-                                 kRMaxSlots);
+      const int held = resident_held_bytes(cfg->kx, c->geo.xbits);
+      auto slots_for = [&](int held_bytes) {
+        return std::min(((int)max_smem - kRHeadBytes - estages * (resident_stage_bytes(wm) + held_bytes)) / kRSlotBytes,
+                        kRMaxSlots);
+      };
+      const int slots = slots_for(0);
       // a pair may give a CTA at most slots - 2 tiles: the rest of the ring lets the load side
       // run ahead into the next pair while this one is quantized and stored
       const int spare = 2;
@@ -601,13 +607,18 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
         build_resident((long long)c->sm_count * (slots - spare), o.test_missing_tiles, &c->geo);
         c->res_slots = slots;
         c->res_estages = estages;
-        c->res_smem = resident_smem_bytes(slots, estages, wm);
-        bool fits = !c->geo.rtiles.empty();
+        c->res_smem = resident_smem_bytes(slots, estages, wm, 0);
+        // with the l2 term one slot less (two for unquantized weights): still as many as the largest
+        // pair gives a CTA, so the loads of a pair never wait for its own stores
+        c->res_slots_l2 = slots_for(held);
+        c->res_smem_l2 = resident_smem_bytes(c->res_slots_l2, estages, wm, held);
+        bool fits = !c->geo.rtiles.empty() && c->res_slots_l2 >= slots - spare;
         for (int variant = 0; variant < 3 && fits; ++variant) {          // plain + words, plain, l2
           WorkerResidentKernel k = pick_worker_resident(c, variant == 2, variant == 0);
           int per_sm = 0;
-          fits = cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->res_smem)) &&
-                 cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kRThreads, c->res_smem)) &&
+          const size_t smem = variant == 2 ? c->res_smem_l2 : c->res_smem;
+          fits = cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) &&
+                 cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kRThreads, smem)) &&
                  per_sm >= 1;
         }
         if (fits)
@@ -742,14 +753,16 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
       rp.done = c->d_done;
       rp.TR = (int)c->geo.rtiles.size();
       rp.total = (long long)worker_count * rp.TR;
-      rp.slots = c->res_slots;
+      rp.slots = l2 ? c->res_slots_l2 : c->res_slots;
       rp.estages = c->res_estages;
+      rp.held_bytes = l2 ? resident_held_bytes(c->cfg.kx, c->geo.xbits) : 0;
       void* args[] = {&rp};
       cudaError_t e;
       {
         LaunchTimer lt(c, QADAM_K_WORKER_FUSED);
         e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(pick_worker_resident(c, l2, use_words)),
-                                        dim3(c->grid_resident), dim3(kRThreads), args, c->res_smem, c->stream);
+                                        dim3(c->grid_resident), dim3(kRThreads), args, l2 ? c->res_smem_l2 : c->res_smem,
+                                        c->stream);
       }
       if (cuda_ok(e)) {
         c->launches += 1;

@@ -148,11 +148,35 @@ __device__ __forceinline__ void add_l2_term_held(const WorkerParams& p, long lon
   for (int c = 0; c < 4; ++c) gg[c] = __fadd_rn(gg[c], __fmul_rn(p.lambda, w[c]));
 }
 
-// The same from codes fetched earlier with held_fetch8.
-__device__ __forceinline__ void add_l2_term_fetched(const WorkerParams& p, int lane, unsigned lo, unsigned hi,
-                                                    float gg[4]) {
+// The same from a copy of the tile's held weights in shared memory (packed codes, or x itself);
+// row: the row's first element in the tile.
+__device__ __forceinline__ void add_l2_term_staged(const WorkerParams& p, const unsigned char* held, int row, int lane,
+                                                   float gg[4]) {
   float w[4];
-  held_decode8(p, lane, lo, hi, w);
+  if (p.kx < 0) {
+    const float4 v = *reinterpret_cast<const float4*>(held + (row + lane * 4) * 4);
+    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+  } else {
+    const unsigned* words = reinterpret_cast<const unsigned*>(held + row / 8 * p.xbits);
+    if (p.xbits <= 8) {
+      const int F = 4 * p.xbits, i = (F * lane) >> 5;
+      const unsigned lo = words[i], hi = ((F * lane) & 31) + F > 32 ? words[i + 1] : 0u;
+      held_decode8(p, lane, lo, hi, w);
+    } else {
+      const int half = 2 * p.xbits;                     // two codes, at most 32 bits
+      const unsigned mask = (1u << p.xbits) - 1u;
+      const float step = exp2i(-(p.kx + 1));
+      const float bias = -(8388608.0f + (float)(1 << p.kx));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int bit = (2 * lane + h) * half, i = bit >> 5;
+        const unsigned hi = (bit & 31) + half > 32 ? words[i + 1] : 0u;
+        const unsigned f = __funnelshift_r(words[i], hi, bit & 31);
+        w[2 * h] = __fmul_rn(__fadd_rn(__uint_as_float(0x4b000000u | (f & mask)), bias), step);
+        w[2 * h + 1] = __fmul_rn(__fadd_rn(__uint_as_float(0x4b000000u | ((f >> p.xbits) & mask)), bias), step);
+      }
+    }
+  }
 #pragma unroll
   for (int c = 0; c < 4; ++c) gg[c] = __fadd_rn(gg[c], __fmul_rn(p.lambda, w[c]));
 }

@@ -80,6 +80,7 @@ struct WorkerResidentParams {
   int TR;                 // resident tiles per worker
   int slots;              // slots of the CTA's ring (a pair gives a CTA fewer tiles than this)
   int estages;            // stages of the e ring
+  int held_bytes;         // l2 term: bytes of a tile's held weights, which a stage then carries too
 };
 
 // 24 consumer warps, split between the two sides by where the arithmetic is: with the
@@ -87,8 +88,9 @@ struct WorkerResidentParams {
 // thread and tile) and the store side quantizes (16 warps, 2 rows); with the moments on
 // the workers the load side also runs the moment updates, a root and a division per
 // element (16 warps) and the store side gets 8; the same 16 / 8 split serves the l2 term,
-// whose decode of the held weights is load-side work (measured: 3.59 -> 3.28 ms on the
-// BERT-shaped set, while without the term 8 / 16 stays the faster split).
+// whose decode of the held weights is load-side work.  The held weights of a tile come with
+// its stage (a bulk copy of the packed codes, or of x): read from global memory where they are
+// used, their latency was paid once per tile.
 constexpr int kRColThreads = 256;       // threads across a 1024-element row, 4 elements each
 constexpr int kRConsumerWarps = 24;
 constexpr int kRRoleWarp0 = kRConsumerWarps;      // producer, publisher, dispatcher follow
@@ -109,7 +111,6 @@ struct RLoadHeader {       // one per tile in flight on the load side (ring of k
                            // is handed over inside the CTA (nothing to publish or to count)
   unsigned max_bits;       // max |u| of the tile, folded in by the consumer warps
   long long elem;          // worker * D + first element: where m, v go back (moments on the workers)
-  long long off;           // first element in the vector: where the held weights are (l2 term)
 };
 struct RCommand {          // one per quantize command
   long long off;           // first element (padded layout)
@@ -136,12 +137,15 @@ static_assert(sizeof(RSmem) <= kRHeadBytes, "head of the shared-memory layout");
 __host__ __device__ constexpr int resident_stage_bytes(bool worker_moments) {
   return (worker_moments ? 3 : 1) * kRSlotBytes;
 }
-__host__ __device__ inline size_t resident_smem_bytes(int slots, int estages, bool worker_moments) {
-  return kRHeadBytes + (size_t)slots * kRSlotBytes + (size_t)estages * resident_stage_bytes(worker_moments);
+__host__ __device__ inline size_t resident_smem_bytes(int slots, int estages, bool worker_moments, int held_bytes) {
+  return kRHeadBytes + (size_t)slots * kRSlotBytes +
+         (size_t)estages * (resident_stage_bytes(worker_moments) + held_bytes);
 }
+// With the l2 term a stage also carries the tile's held weights: b_x bits (x: 32) per element.
+__host__ __device__ constexpr int resident_held_bytes(int kx, int xbits) { return kTileElems / 8 * (kx < 0 ? 32 : xbits); }
 
 // MODE: grid of Q_g; WM: moments on the workers; L2: the l2 term lambda * (held weights) is
-// added to g first (the held weights are decoded from the packed broadcast, or read from x);
+// added to g first (the held weights come with the stage);
 // WORDS: the hand-over goes through one word per (pair, CTA) (rp.words) instead of one
 // counter per pair (rp.done) and atomics.
 template <int MODE, bool WM, bool L2, bool WORDS>
@@ -155,6 +159,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
   RSmem* ps = reinterpret_cast<RSmem*>(smem_raw);
   unsigned char* slot_base = smem_raw + kRHeadBytes;
   unsigned char* ering_base = slot_base + (size_t)rp.slots * kRSlotBytes;
+  unsigned char* held_base = ering_base + (size_t)rp.estages * kStageBytes;     // l2 term only
   const WorkerParams& p = rp.w;
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
@@ -219,9 +224,10 @@ worker_resident_kernel(const WorkerResidentParams rp) {
           const unsigned bytes = (unsigned)cur.count * 4u;
           const long long eo = (long long)(p.worker_begin + worker) * p.D + cur.off;
           hd->elem = eo;
-          hd->off = cur.off;
           unsigned char* st = ering_base + (size_t)s * kStageBytes;
-          mbar_arrive_expect_tx(&ps->e_full[s], (WM ? 4u : 2u) * bytes);
+          const int hbits = p.kx < 0 ? 32 : p.xbits;               // l2 term: bits of a held weight
+          const unsigned hbytes = L2 ? (unsigned)(cur.count / 8 * hbits) : 0u;
+          mbar_arrive_expect_tx(&ps->e_full[s], (WM ? 4u : 2u) * bytes + hbytes);
           bulk_load(slot_base + (size_t)slot * kRSlotBytes, p.g + (long long)worker * p.D + cur.off, bytes,
                     &ps->e_full[s]);
           bulk_load(st, p.e + eo, bytes, &ps->e_full[s]);
@@ -229,6 +235,10 @@ worker_resident_kernel(const WorkerResidentParams rp) {
             bulk_load(st + kRSlotBytes, p.m + eo, bytes, &ps->e_full[s]);
             bulk_load(st + 2 * kRSlotBytes, p.v + eo, bytes, &ps->e_full[s]);
           }
+          if constexpr (L2)       // tile starts are multiples of 128 elements: 16-byte aligned at any width
+            bulk_load(held_base + (size_t)s * rp.held_bytes,
+                      (p.kx < 0 ? reinterpret_cast<const unsigned char*>(p.x) : p.wcodes) + cur.off / 8 * hbits, hbytes,
+                      &ps->e_full[s]);
         }
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -422,49 +432,18 @@ worker_resident_kernel(const WorkerResidentParams rp) {
     const int row0 = tid / kRColThreads;
     int s = 0;
     unsigned ph = 0;
-    // l2 term with packed weights of at most 8 bits: the code words of a tile are fetched
-    // while the tile before it is processed (and the descriptor of the tile after it is
-    // read), so that their latency stays off the path.  hw_*: words of the tile about to be
-    // processed, one pair per row of this thread.
     constexpr int kMineL = kRows / kLRowStep;
-    // (With the moments on the workers the 16 load-side warps hide that latency themselves,
-    // and the extra registers cost more than the fetch ahead gains: measured.)
-    const bool pref = L2 && !WM && p.kx >= 0 && p.xbits <= 8;
-    unsigned hw_lo[kMineL], hw_hi[kMineL];
-    int pj = my_tiles > 0 ? (int)((long long)cta % rp.TR) : 0;      // index of the tile whose descriptor is in `ahead`
-    RTile ahead = RTile{0, 0, 0, 0, 0};
-    auto step_j = [&]() { pj += ctas; while (pj >= rp.TR) pj -= rp.TR; };
-    auto fetch_rows = [&](const RTile& t, unsigned (&lo)[kMineL], unsigned (&hi)[kMineL]) {
-#pragma unroll
-      for (int r = 0; r < kMineL; ++r) {
-        const int q = row0 + r * kLRowStep;
-        lo[r] = hi[r] = 0u;
-        if (q * kRowElems + gt * 4 < t.count)
-          held_fetch8(p, t.off + q * kRowElems + (gt >> 5) * 128, lane, lo[r], hi[r]);
-      }
-    };
-    if (pref && my_tiles > 0) {
-      fetch_rows(rp.rtiles[pj], hw_lo, hw_hi);                       // tile 0
-      step_j();
-      if (my_tiles > 1) ahead = rp.rtiles[pj];                       // descriptor of tile 1
-    }
     for (long long i = 0; i < my_tiles; ++i) {
-      unsigned nx_lo[kMineL], nx_hi[kMineL];
-      if (pref && i + 1 < my_tiles) {
-        fetch_rows(ahead, nx_lo, nx_hi);                             // words of tile i + 1
-        step_j();
-        if (i + 2 < my_tiles) ahead = rp.rtiles[pj];                 // descriptor of tile i + 2
-      }
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&ps->e_full[s], ph, abort_flag, p.status, spin))) break;
       RLoadHeader* hdp = &ps->load_hd[i & (kRHeaders - 1)];
       const int slot = hdp->slot, count = hdp->count;
       float* su = reinterpret_cast<float*>(slot_base + (size_t)slot * kRSlotBytes) + gt * 4;
       const float* se = reinterpret_cast<const float*>(ering_base + (size_t)s * kStageBytes) + gt * 4;
+      const unsigned char* held = L2 ? held_base + (size_t)s * rp.held_bytes : nullptr;
       unsigned mx = 0;
       if constexpr (WM) {
         // Algorithm 3: v, m updates, u = alpha m / sqrt(v + eps) + e; m, v go straight back
         const long long elem = hdp->elem;
-        const long long off = hdp->off;
         float4 g4[kRows / kLRowStep], e4[kRows / kLRowStep], m4[kRows / kLRowStep], v4[kRows / kLRowStep];
 #pragma unroll
         for (int r = 0; r < kRows / kLRowStep; ++r) {
@@ -482,10 +461,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
           if (q * kRowElems + gt * 4 >= count) continue;               // warp-uniform
           float gg[4] = {g4[r].x, g4[r].y, g4[r].z, g4[r].w};
           float ee[4] = {e4[r].x, e4[r].y, e4[r].z, e4[r].w};
-          if constexpr (L2) {
-            if (pref) add_l2_term_fetched(p, lane, hw_lo[r], hw_hi[r], gg);
-            else add_l2_term(p, off + q * kRowElems + (gt >> 5) * 128, lane, gg);
-          }
+          if constexpr (L2) add_l2_term_staged(p, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
           float mm[4] = {m4[r].x, m4[r].y, m4[r].z, m4[r].w};
           float vs[4] = {v4[r].x, v4[r].y, v4[r].z, v4[r].w};
           float uu[4];
@@ -508,10 +484,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
             const float4 g4 = *reinterpret_cast<const float4*>(su + q * kRowElems);
             const float4 e4 = *reinterpret_cast<const float4*>(se + q * kRowElems);
             float gg[4] = {g4.x, g4.y, g4.z, g4.w};
-            if constexpr (L2) {
-              if (pref) add_l2_term_fetched(p, lane, hw_lo[r], hw_hi[r], gg);
-              else add_l2_term(p, hdp->off + q * kRowElems + (gt >> 5) * 128, lane, gg);
-            }
+            if constexpr (L2) add_l2_term_staged(p, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
             const float4 u4 = make_float4(__fadd_rn(gg[0], e4.x), __fadd_rn(gg[1], e4.y), __fadd_rn(gg[2], e4.z),
                                           __fadd_rn(gg[3], e4.w));
             *reinterpret_cast<float4*>(su + q * kRowElems) = u4;
@@ -528,10 +501,6 @@ worker_resident_kernel(const WorkerResidentParams rp) {
       if (lane == 0) {
         mbar_arrive(&ps->e_empty[s]);                            // the stage has been read: it can be refilled
         mbar_arrive(&ps->hd_ready[i & (kRHeaders - 1)]);         // the header's maximum is complete
-      }
-      if constexpr (L2) {
-#pragma unroll
-        for (int r = 0; r < kMineL; ++r) { hw_lo[r] = nx_lo[r]; hw_hi[r] = nx_hi[r]; }
       }
       if (++s == estages) { s = 0; ph ^= 1u; }
     }
