@@ -73,7 +73,7 @@ struct Geometry {
   std::vector<RTile> rtiles;
   std::vector<Tile> btiles;
   long long resident_elems = 0;      // padded elements of the resident segments (one vector)
-  size_t off_rtiles = 0, off_btiles = 0, off_words = 0, off_deferred = 0;
+  size_t off_rtiles = 0, off_btiles = 0, off_words = 0, off_epoch = 0, off_deferred = 0;
   size_t words_bytes = 0;            // room for the per-(pair, CTA) words of the on-chip worker kernel
 };
 
@@ -193,6 +193,8 @@ int build_geometry(const qadam_config* c, Geometry* g) {
     const size_t want = (size_t)c->n * c->num_segments * kWordCtas * sizeof(unsigned long long);
     g->words_bytes = want <= kWordBudget ? want : 0;
     wo += (size_t)round_up64((int64_t)g->words_bytes, 256);
+    g->off_epoch = wo;
+    wo += 256;
   }
   // flags of the rows the sweep leaves to the second kernel (1 / 8192 of the size of e)
   g->off_deferred = wo;
@@ -237,6 +239,7 @@ struct qadam_ctx {
   RTile* d_rtiles = nullptr;
   Tile* d_btiles = nullptr;
   unsigned char* d_deferred = nullptr;
+  unsigned* d_epoch = nullptr;
   unsigned long long* d_words = nullptr;   // nullptr: one counter per pair instead
   // qadam_step_host: the copy of worker i + 1 runs on a stream of its own while worker i is compressed
   cudaStream_t copy_stream = nullptr;
@@ -348,11 +351,12 @@ PipeKernel pick_pipe(const qadam_ctx* c) {
 
 using WorkerResidentKernel = void (*)(const WorkerResidentParams);
 
-// With the l2 term the counter hand-over runs (the words were measured slower there).
 template <int MODE>
 WorkerResidentKernel pick_worker_resident_mode(bool worker_moments, bool l2, bool words) {
-  if (l2) return worker_moments ? worker_resident_kernel<MODE, true, true, false>
-                                : worker_resident_kernel<MODE, false, true, false>;
+  if (l2 && worker_moments) return words ? worker_resident_kernel<MODE, true, true, true>
+                                         : worker_resident_kernel<MODE, true, true, false>;
+  if (l2) return words ? worker_resident_kernel<MODE, false, true, true>
+                       : worker_resident_kernel<MODE, false, true, false>;
   if (worker_moments) return words ? worker_resident_kernel<MODE, true, false, true>
                                    : worker_resident_kernel<MODE, true, false, false>;
   return words ? worker_resident_kernel<MODE, false, false, true>
@@ -517,6 +521,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     c->d_rtiles = reinterpret_cast<RTile*>(ws + c->geo.off_rtiles);
     c->d_btiles = reinterpret_cast<Tile*>(ws + c->geo.off_btiles);
     c->d_deferred = ws + c->geo.off_deferred;
+    c->d_epoch = reinterpret_cast<unsigned*>(ws + c->geo.off_epoch);
     c->d_words = c->geo.words_bytes ? reinterpret_cast<unsigned long long*>(ws + c->geo.off_words) : nullptr;
   }
 
@@ -613,10 +618,10 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
         c->res_slots_l2 = slots_for(held);
         c->res_smem_l2 = resident_smem_bytes(c->res_slots_l2, estages, wm, held);
         bool fits = !c->geo.rtiles.empty() && c->res_slots_l2 >= slots - spare;
-        for (int variant = 0; variant < 3 && fits; ++variant) {          // plain + words, plain, l2
-          WorkerResidentKernel k = pick_worker_resident(c, variant == 2, variant == 0);
+        for (int variant = 0; variant < 4 && fits; ++variant) {          // without and with the l2 term, counters and words
+          WorkerResidentKernel k = pick_worker_resident(c, variant >= 2, (variant & 1) != 0);
           int per_sm = 0;
-          const size_t smem = variant == 2 ? c->res_smem_l2 : c->res_smem;
+          const size_t smem = variant >= 2 ? c->res_smem_l2 : c->res_smem;
           fits = cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) &&
                  cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kRThreads, smem)) &&
                  per_sm >= 1;
@@ -641,6 +646,11 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
         (!c->geo.btiles.empty() &&
          !cuda_ok(cudaMemcpyAsync(c->d_btiles, c->geo.btiles.data(), c->geo.btiles.size() * sizeof(Tile),
                                   cudaMemcpyHostToDevice, c->stream))))) ||
+      // launches of the on-chip worker kernel count from 1, words of launch 0 are empty
+      (c->grid_resident > 0 && c->d_words != nullptr &&
+       (!cuda_ok(cudaMemsetAsync(c->d_words, 0, c->geo.words_bytes, c->stream)) ||
+        !cuda_ok(cudaMemsetAsync(c->d_epoch, 0, 2 * sizeof(unsigned), c->stream)) ||
+        !cuda_ok(cudaMemsetAsync(c->d_epoch, 1, 1, c->stream)))) ||
       !cuda_ok(cudaMemsetAsync(b->status, 0, sizeof(uint32_t), c->stream)) ||
       !cuda_ok(cudaStreamSynchronize(c->stream))) {
     delete c; return QADAM_ERR_CUDA;
@@ -732,23 +742,24 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
     if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
     c->launches += 1;
   } else {
-    // the scales of these workers start at zero (the kernels fold maxima into them)
-    if (!cuda_ok(cudaMemsetAsync(p.scale_bits + (size_t)worker_begin * p.S, 0,
-                                 sizeof(unsigned) * (size_t)worker_count * p.S, c->stream)))
-      return QADAM_ERR_CUDA;
     bool on_chip = c->grid_resident > 0;
+    const bool l2 = c->lambda != 0.0f;
+    const bool use_words = on_chip && c->d_words != nullptr && c->grid_resident <= kWordCtas &&
+                           c->opt.hand_over == QADAM_HANDOVER_AUTO;
+    // kernels that fold maxima into the scales need these workers' at zero; the on-chip kernel
+    // with words stores each once
+    auto clear_scales = [&]() {
+      return cuda_ok(cudaMemsetAsync(p.scale_bits + (size_t)worker_begin * p.S, 0,
+                                     sizeof(unsigned) * (size_t)worker_count * p.S, c->stream));
+    };
+    if ((!use_words || !c->geo.btiles.empty()) && !clear_scales()) return QADAM_ERR_CUDA;
     if (on_chip) {
-      const size_t pairs = (size_t)c->cfg.n * p.S;     // all pairs' records are cleared, the call's are used
-      const bool l2 = c->lambda != 0.0f;
-      const bool use_words = !l2 && c->d_words != nullptr && c->grid_resident <= kWordCtas &&
-                             c->opt.hand_over == QADAM_HANDOVER_AUTO;
-      if (!cuda_ok(cudaMemsetAsync(c->d_done, 0, sizeof(unsigned) * pairs, c->stream)) ||
-          (use_words && !cuda_ok(cudaMemsetAsync(c->d_words, 0, sizeof(unsigned long long) * pairs * c->grid_resident,
-                                                 c->stream))))
+      if (!use_words && !cuda_ok(cudaMemsetAsync(c->d_done, 0, sizeof(unsigned) * (size_t)c->cfg.n * p.S, c->stream)))
         return QADAM_ERR_CUDA;
       WorkerResidentParams rp;
       rp.w = p;
       rp.words = use_words ? c->d_words : nullptr;
+      rp.epoch = c->d_epoch;
       rp.rtiles = c->d_rtiles;
       rp.done = c->d_done;
       rp.TR = (int)c->geo.rtiles.size();
@@ -776,6 +787,7 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
         // nothing of it runs, and the streaming launches over the whole vector still can
         (void)cudaGetLastError();
         on_chip = false;
+        if (use_words && c->geo.btiles.empty() && !clear_scales()) return QADAM_ERR_CUDA;
       }
     }
     if (!on_chip) {

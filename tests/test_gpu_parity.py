@@ -321,6 +321,50 @@ def test_on_chip_worker_one_tile_pairs(placement, hand_over):
 
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
+def test_on_chip_worker_words_of_earlier_launches_do_not_count(placement):
+    # the words that carry a pair's scale between CTAs are not cleared between launches: a launch
+    # tells its own by a number that the device counts up, so calls for some workers only, calls
+    # with the l2 term in between and replays of a captured step must all agree with the oracle
+    import paper_2004_14180_b200 as qb
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    seg = [sms * 2 * 4096 + 300, 5000, 64, 70000, 129]
+    n, d = 3, sum(seg)
+    rng = np.random.default_rng(300 + placement)
+    x1 = (rng.standard_normal(d) * 0.2).astype(np.float32)
+    p = Pair(seg, n, 0, 0, placement, x1=x1)
+    for t in range(6):
+        p.set_regularization(5e-4 if t % 3 == 1 else 0.0)
+        # smaller gradients every step: a maximum left from the step before would be too large
+        p.step(_rand_grads(rng, n, d, 0.1 ** t), split_workers=t % 2 == 1)
+        p.compare_state()
+    p.close()
+
+    stream = torch.cuda.Stream()
+    q = qb.QAdam(seg, n, kg=0, kx=0, placement=placement, x1=torch.from_numpy(x1), stream=stream)
+    import oracle
+    c = oracle.OracleState(seg, n, 0, 0, placement, 0.9, 0.999, 1e-8)
+    c.set_weights(x1)
+    g = c.to_padded(_rand_grads(rng, n, d))
+    g_dev = torch.from_numpy(g).cuda()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        q.step(1, g_dev)
+    for scale in (1.0, 1e-2, 1e-4):
+        g_dev.copy_(torch.from_numpy(g * np.float32(scale)))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        c.step(g * np.float32(scale), 1e-3)
+        assert np.array_equal(q.gcodes.cpu().numpy(), c.gcodes)
+        for name in ("scales", "x", "m", "v", "e"):
+            assert bits_equal(getattr(q, name).cpu().numpy(), getattr(c, name)), name
+    assert q.poll_status() == 0
+    del graph
+    q.close()
+
+
+@pytest.mark.parametrize("placement", [S_MODE, W_MODE])
 def test_streaming_launches_only(placement):
     # worker_kernel = STREAMING sends every pair through the two streaming launches, the
     # route that otherwise only pairs too large for the chip, partial worker ranges and some
