@@ -587,6 +587,35 @@ def test_pipelined_server_code_densities(density, placement):
         p.close()
 
 
+# ---------------------------------------------------------------- averages over any number of workers
+
+@pytest.mark.parametrize("kg,grid", [(0, 0), (1, 0), (3, 1)])
+@pytest.mark.parametrize("n", [3, 7, 12, 24, 63])
+def test_average_over_worker_counts_that_are_not_powers_of_two(n, kg, grid):
+    # sum / n without a division, for scales of ordinary size, with it for the others: segments of
+    # ordinary magnitudes, of workers that cancel each other (sums of 0 and near 0), and on either
+    # side of 2^-60, down to subnormals; the other limit, 2^100, by the step size with the moments
+    # on the workers (on the server the second moment of such a gradient is not finite)
+    seg = [9000, 4096, 2500, 2500, 640]
+    mags = [1e-2, 1.0, 2.0 ** -59, 2.0 ** -61, 1e-42]
+    rng = np.random.default_rng(4000 + n)
+    d = sum(seg)
+    x1 = (rng.standard_normal(d) * 0.2).astype(np.float32)
+    on_workers = Pair(seg, n, kg, 0, W_MODE, x1=x1, grid_g=grid)
+    on_server = Pair(seg, n, kg, 0, S_MODE, x1=x1, grid_g=grid)
+    for t, lr in enumerate((1e-3, 2.0 ** 97, 2.0 ** 101)):
+        g = rng.standard_normal((n, d)).astype(np.float32)
+        g *= rng.random((n, d)) < (0.02 if t == 1 else 1.0)
+        g *= np.concatenate([np.full(l, m) for l, m in zip(seg, mags)]).astype(np.float32)
+        g[1::2, 9000:9000 + 4096] = -g[:n - n % 2:2, 9000:9000 + 4096]
+        on_workers.step(g, lr=lr)
+        on_workers.compare_state()
+        on_server.step(g)
+        on_server.compare_state()
+    on_workers.close()
+    on_server.close()
+
+
 # ---------------------------------------------------------------- the stochastic ternary operator
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])

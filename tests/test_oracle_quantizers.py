@@ -216,3 +216,18 @@ def test_two_bit_packing_against_numpy_bit_order(oracle):
     codes = rng.integers(0, 3, 4096).astype(np.uint32)
     bits = np.stack([(codes >> 0) & 1, (codes >> 1) & 1], axis=1).astype(np.uint8).reshape(-1)
     assert np.array_equal(oracle.pack_bits(codes, 2), np.packbits(bits, bitorder="little"))
+
+
+@pytest.mark.parametrize("n", [3, 5, 6, 7, 11, 12, 24, 31, 37, 48, 63])
+def test_division_by_an_integer_from_its_rounded_reciprocal(n):
+    """The server pass divides a sum by n as q = fl(a inv), r = fl(a - n q), fl(q + r inv) with
+    inv = fl(1 / n): equal to fl(a / n) for every significand (the exponent does not matter away
+    from the ends of the range).  The fused operations are formed in binary64, where a - n q is
+    exact and q + r inv is not a near-tie of binary32 (a / n is at least 1 / 128 ulp from one)."""
+    f = np.float32
+    a = (np.arange(1 << 23, dtype=np.uint32) | np.uint32(0x3f800000)).view(f)
+    inv = f(1) / f(n)
+    q = a * inv
+    r = (a.astype(np.float64) - np.float64(n) * q).astype(f)
+    got = (q.astype(np.float64) + r.astype(np.float64) * np.float64(inv)).astype(f)
+    assert np.array_equal(got, a / f(n))
