@@ -58,6 +58,11 @@ int grad_levels(int kg, int grid) {
 constexpr int kWordCtas = 256;                       // CTAs the per-pair words are sized for
 constexpr size_t kWordBudget = (size_t)32 << 20;     // bytes of workspace they may take
 
+// Elements from which the stochastic operator runs on chip: one pass over g, e against two
+// (ResNet-shaped, n = 8: 405 -> 255 us; 4.0 x 10^6 elements, n = 8: 152 -> 103).  Below it both
+// are a few microseconds of latency, and the streaming launches need no cooperative launch.
+constexpr int64_t kStochasticOnChip = 1 << 20;
+
 struct Geometry {
   std::vector<int64_t> seg_len, seg_off;
   int64_t D = 0;
@@ -368,6 +373,7 @@ WorkerResidentKernel pick_worker_resident(const qadam_ctx* c, bool l2, bool word
   switch (c->geo.gmode) {
     case G_TERNARY: return pick_worker_resident_mode<G_TERNARY>(w, l2, words);
     case G_FIVE:    return pick_worker_resident_mode<G_FIVE>(w, l2, words);
+    case G_STOCHASTIC: return pick_worker_resident_mode<G_STOCHASTIC>(w, l2, words);
     case G_POW2:    return pick_worker_resident_mode<G_POW2>(w, l2, words);
     default:        return pick_worker_resident_mode<G_UNIFORM>(w, l2, words);
   }
@@ -592,8 +598,9 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     int coop = 0, max_smem = 0;
     const bool want_split = o.worker_kernel == QADAM_WORKER_STREAMING;
     const bool wm = cfg->placement == QADAM_PLACE_WORKER;
-    // (the stochastic operator runs in the streaming launches only)
-    const bool eligible = !want_split && c->geo.gmode != G_IDENTITY && c->geo.gmode != G_STOCHASTIC &&
+    // the stochastic operator in short vectors stays with the two streaming launches: see kStochasticOnChip
+    const bool eligible = !want_split && c->geo.gmode != G_IDENTITY &&
+        (c->geo.gmode != G_STOCHASTIC || c->geo.D >= kStochasticOnChip) &&
         cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) && coop &&
         cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     if (eligible) {

@@ -117,7 +117,7 @@ __device__ __forceinline__ float level_value(int c, int k) {
 // the division gives.
 struct GradScale {
   float s;
-  float inv;      // fl(1 / s), times 2^k for the uniform grid
+  float inv;      // fl(1 / s), times 2^k for the uniform grid, times 2^24 for the stochastic operator
   float half;     // ternary: s / 2 (exact) and the upper end of the sliver above it
   float half_hi;
   bool fast;      // s is an ordinary number (not zero, tiny, Inf or NaN): the fast paths apply
@@ -130,6 +130,9 @@ __device__ __forceinline__ GradScale grad_scale(float s, int k) {
   g.half = __fmul_rn(0.5f, s);
   g.half_hi = __fmul_rn(g.half, 1.000000476837158203125f);          // 1 + 2^-21
   g.inv = 0.0f;
+  if constexpr (MODE == G_STOCHASTIC) {
+    if (g.fast) g.inv = __fdiv_rn(16777216.0f, s);
+  }
   if constexpr (MODE == G_FIVE || MODE == G_POW2 || MODE == G_UNIFORM) {
     if (g.fast) {
       g.inv = __fdiv_rn(1.0f, s);
@@ -348,6 +351,44 @@ __device__ __forceinline__ unsigned quantize_grad_stochastic(float u, float s, u
   const float deq = one ? (neg ? -s : s) : 0.0f;
   e_next = __fsub_rn(u, deq);
   return one ? (neg ? 0u : 2u) : 1u;
+}
+
+// The same for 4 consecutive coordinates of one lane: the error update and the lane's byte of
+// packed codes.  r < y is i < 2^24 y with i = word >> 8, and y' = fl(|u| fl(2^24 / s)) is within 2^-22
+// (relative) of 2^24 y, so i against y' (1 -+ 2^-21) settles it but for a band that one coordinate
+// in a million falls into; there, and for i = 0 (where a y too small for the estimate could
+// matter), the division decides for the lane's four coordinates.
+__device__ __forceinline__ unsigned quantize_stochastic4(const float (&u)[4], const GradScale& gs, const uint4& words,
+                                                         float (&e_next)[4]) {
+  const unsigned w[4] = {words.x, words.y, words.z, words.w};
+  float up[4];
+  bool divide = !gs.fast;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float i = (float)(w[c] >> 8);
+    const float yp = __fmul_rn(fabsf(u[c]), gs.inv);
+    const bool below = i < __fmul_rn(yp, 0.99999952316284179688f);         // 1 - 2^-21
+    const bool near = i < __fmul_rn(yp, 1.00000047683715820313f);          // 1 + 2^-21
+    up[c] = below ? 1.0f : 0.0f;
+    divide = divide || below != near || i == 0.0f;
+  }
+  unsigned byte;
+  if (divide) {
+    byte = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) byte |= quantize_grad_stochastic(u[c], gs.s, w[c], e_next[c]) << (2 * c);
+  } else {
+    float cf[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float sign1 = __uint_as_float((__float_as_uint(u[c]) & 0x80000000u) | 0x3f800000u);   // +-1 with u's sign
+      e_next[c] = __fsub_rn(u[c], __fmaf_rn(up[c], __fmul_rn(sign1, gs.s), 0.0f));
+      cf[c] = __fmaf_rn(up[c], sign1, 1.0f);
+    }
+    const float packed = __fmaf_rn(__fmaf_rn(__fmaf_rn(cf[3], 4.0f, cf[2]), 4.0f, cf[1]), 4.0f, cf[0]);
+    byte = __float_as_uint(__fadd_rn(packed, 8388608.0f)) & 0xffu;
+  }
+  return byte;
 }
 
 // One coordinate of Q_x (Section 5.1): nearest point of the grid c / 2^(kx+1),

@@ -636,7 +636,7 @@ worker_quantize_kernel(const WorkerParams p) {
       const int w = p.worker_begin + wl[a];
       const unsigned sb = p.scale_bits[(long long)w * p.S + tile[a].seg];
       const float s = __uint_as_float(sb);
-      const GradScale gs = grad_scale<MODE == G_STOCHASTIC ? G_TERNARY : MODE>(s, p.k);
+      const GradScale gs = grad_scale<MODE>(s, p.k);
       if (sb >= 0x7f800000u && threadIdx.x == 0) atomicOr(p.status, 1u);
       const long long so = (long long)w * p.D + tile[a].off;
       unsigned char* cw = p.gcodes + (long long)w * p.gcode_bytes;
@@ -663,10 +663,7 @@ worker_quantize_kernel(const WorkerParams p) {
           const unsigned long long block = (unsigned long long)(tile[a].off + idx) >> 2;
           const uint4 rnd = philox4x32_10(make_uint4((unsigned)block, (unsigned)(block >> 32), (unsigned)w, p.step),
                                           make_uint2(p.seed_lo, p.seed_hi));
-          code[0] = quantize_grad_stochastic(uu[0], s, rnd.x, en[0]);
-          code[1] = quantize_grad_stochastic(uu[1], s, rnd.y, en[1]);
-          code[2] = quantize_grad_stochastic(uu[2], s, rnd.z, en[2]);
-          code[3] = quantize_grad_stochastic(uu[3], s, rnd.w, en[3]);
+          code[0] = quantize_stochastic4(uu, gs, rnd, en);   // the lane's byte of four codes
         } else if constexpr (MODE == G_TERNARY) {
           code[0] = quantize_ternary4(uu, gs, en);           // the lane's byte of four codes
         } else if constexpr (MODE == G_FIVE) {
@@ -678,10 +675,8 @@ worker_quantize_kernel(const WorkerParams p) {
         st_f4(p.e + so + idx, make_float4(en[0], en[1], en[2], en[3]));
         const long long row_elem = tile[a].off + r * kRowElems + warp * 128;
         void* dst = cw + row_elem * p.bits / 8;
-        if constexpr (MODE == G_TERNARY) {
+        if constexpr (MODE == G_TERNARY || MODE == G_STOCHASTIC) {
           store_row_of_code_bytes(code[0], dst, lane);
-        } else if constexpr (MODE == G_STOCHASTIC) {
-          pack_row_store<2>(code[0], code[1], code[2], code[3], dst, lane);
         } else if constexpr (MODE == G_FIVE) {
           pack_row_store_fields<3>(code[0], dst, lane);
         } else {

@@ -547,7 +547,14 @@ worker_resident_kernel(const WorkerResidentParams rp) {
         const float uu[4] = {u4[r].x, u4[r].y, u4[r].z, u4[r].w};
         unsigned code[4];
         float en[4];
-        if constexpr (MODE == G_TERNARY) {
+        if constexpr (MODE == G_STOCHASTIC) {
+          // the four coordinates of this thread are one block of the stream, see worker_quantize_kernel
+          const unsigned long long block = (unsigned long long)(cd.off + q * kRowElems + gt * 4) >> 2;
+          const uint4 rnd = philox4x32_10(
+              make_uint4((unsigned)block, (unsigned)(block >> 32), (unsigned)cd.worker, p.step),
+              make_uint2(p.seed_lo, p.seed_hi));
+          code[0] = quantize_stochastic4(uu, gs, rnd, en);
+        } else if constexpr (MODE == G_TERNARY) {
           code[0] = quantize_ternary4(uu, gs, en);             // the lane's byte of four codes
         } else if constexpr (MODE == G_FIVE) {
           code[0] = quantize_five4(uu, gs, en);                // the lane's 12 bits of four codes
@@ -558,7 +565,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
         *reinterpret_cast<float4*>(ew + q * kRowElems) = make_float4(en[0], en[1], en[2], en[3]);
         const long long row_elem = cd.off + q * kRowElems + gwarp * 128;
         void* dst = cw + row_elem * p.bits / 8;
-        if constexpr (MODE == G_TERNARY) {
+        if constexpr (MODE == G_TERNARY || MODE == G_STOCHASTIC) {
           store_row_of_code_bytes(code[0], dst, lane);
         } else if constexpr (MODE == G_FIVE) {
           pack_row_store_fields<3>(code[0], dst, lane);

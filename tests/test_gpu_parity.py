@@ -641,6 +641,30 @@ def test_stochastic_ternary_operator(n, seed, placement):
     p.close()
 
 
+@pytest.mark.parametrize("placement", [S_MODE, W_MODE])
+def test_stochastic_ternary_operator_on_chip(placement):
+    # long vectors go through the on-chip kernel: pairs of one tile and of several, a pair beyond the
+    # chip, ragged ends; coins that the estimate of y settles and, with few bits in u / scale,
+    # coins that fall on y itself; a segment of zeros and one of subnormal magnitudes
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    seg = [3 * 4096 + 640, 130, 1, sms * 12 * 4096 + 5, 4096, 2048, 1 << 19]
+    n, d = 2, sum(seg)
+    rng = np.random.default_rng(910 + placement)
+    x1 = (rng.standard_normal(d) * 0.2).astype(np.float32)
+    p = Pair(seg, n, 0, 1, placement, x1=x1, grid_g=2, seed=77)
+    one, two = p.gpu.worker_pass_model()
+    assert one > 0 and two > 0
+    for t, lam in enumerate((0.0, 5e-4)):
+        p.set_regularization(lam)
+        g = _rand_grads(rng, n, d)
+        g[:, -(1 << 19):] = np.round(g[:, -(1 << 19):] * 400) / 4          # few distinct quotients
+        g[:, -(1 << 19) - 2048:-(1 << 19)] = 0.0
+        g[:, -(1 << 19) - 2048 - 4096:-(1 << 19) - 2048] *= np.float32(1e-41)
+        p.step(g)
+        p.compare_state()
+    p.close()
+
+
 def test_stochastic_operator_is_ternary_only():
     import paper_2004_14180_b200 as qb
     with pytest.raises(qb.QAdamError) as ei:
