@@ -543,6 +543,12 @@ __device__ __forceinline__ float2 fma2_rn(float2 a, float2 b, float2 c) {
   return unpack_f2(r);
 }
 
+// Launches of one stream whose second was given the programmatic-serialization attribute: the
+// second may be brought onto SMs that the first has left once all blocks of the first have
+// said so; it waits here until the first has ended and its writes are visible.
+__device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ unsigned warp_max(unsigned v) {
   return __reduce_max_sync(0xffffffffu, v);
 }

@@ -443,6 +443,8 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
     unsigned ph = 0;
     int issued = 0;
     Tile t = my_tiles > 0 ? ptiles[blockIdx.x] : Tile{0, 0, 0};
+    // Everything so far, the tile table included, does not depend on the workers' launch.
+    wait_for_previous_launch();
     for (int j = 0; j < my_tiles; ++j) {
       // next tile's descriptor is fetched while this one is issued
       Tile tn = t;
@@ -517,6 +519,7 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
     // the other waits for its data.  In a tile a thread owns elements 4t..4t+3 of every
     // 1024-element row.  The ring holds a multiple of the group count, so a group steps
     // through its own stages only.
+    wait_for_previous_launch();
     const int group = tid / kPipeGroupThreads;
     const int gt = tid - group * kPipeGroupThreads;           // 0..255
     const int gwarp = gt >> 5;

@@ -186,6 +186,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  let_next_launch_start();                 // the server pass moves in where this kernel's CTAs have left
   volatile int* abort_flag = &ps->abort_flag;
   // the CTA's tiles: t = cta, cta + ctas, ... < total
   const long long my_tiles = cta < rp.total ? (rp.total - cta + ctas - 1) / ctas : 0;
