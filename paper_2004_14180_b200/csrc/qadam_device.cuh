@@ -118,7 +118,7 @@ __device__ __forceinline__ float level_value(int c, int k) {
 struct GradScale {
   float s;
   float inv;      // fl(1 / s), times 2^k for the uniform grid, times 2^24 for the stochastic operator
-  float half;     // ternary: s / 2 (exact) and the upper end of the sliver above it
+  float half;     // ternary: s / 2 (exact) and the upper end of the sliver above it; uniform: s / 2^k
   float half_hi;
   bool fast;      // s is an ordinary number (not zero, tiny, Inf or NaN): the fast paths apply
 };
@@ -136,7 +136,10 @@ __device__ __forceinline__ GradScale grad_scale(float s, int k) {
   if constexpr (MODE == G_FIVE || MODE == G_POW2 || MODE == G_UNIFORM) {
     if (g.fast) {
       g.inv = __fdiv_rn(1.0f, s);
-      if constexpr (MODE == G_UNIFORM) g.inv = __fmul_rn(g.inv, exp2i(k));      // exact
+      if constexpr (MODE == G_UNIFORM) {
+        g.inv = __fmul_rn(g.inv, exp2i(k));      // exact
+        g.half = __fmul_rn(s, exp2i(-k));        // exact
+      }
     }
   }
   return g;
@@ -321,6 +324,46 @@ __device__ __forceinline__ unsigned quantize_five4(const float (&u)[4], const Gr
   return __float_as_uint(__fadd_rn(packed, 8388608.0f)) & 0xfffu;
 }
 
+// Uniform Q_g (levels c / 2^k) of 4 consecutive coordinates of one lane, the error update, and the
+// lane's 4 * bits bits of packed codes (bits = k + 2, at most 8).  Same decisions as
+// quantize_grad<G_UNIFORM>: z' = |u| fl(2^k / s) is within 2^-16 of z = y 2^k, so its nearest integer
+// (by adding and subtracting 1.5 2^23) is the index unless z' lies within 2^-14 of a half, where the
+// division decides for the lane's four coordinates.  On the fp32 pipe like the two above; the
+// dequantized value fl(index s / 2^k) is a multiply-add of +0, so that level 0 gives +0.
+__device__ __forceinline__ unsigned quantize_uniform4(const float (&u)[4], const GradScale& gs, int k, int L, int bits,
+                                                      float (&e_next)[4]) {
+  if (!gs.fast) {
+    unsigned field = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) field |= quantize_grad<G_UNIFORM>(u[c], gs, k, L, e_next[c]) << (c * bits);
+    return field;
+  }
+  float idx[4], worst = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float z = __fmul_rn(fabsf(u[c]), gs.inv);
+    idx[c] = __fsub_rn(__fadd_rn(z, 12582912.0f), 12582912.0f);
+    worst = fmaxf(worst, fabsf(__fsub_rn(z, idx[c])));
+  }
+  if (worst > 0.49993896f) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) idx[c] = (float)level_index<G_UNIFORM>(__fdiv_rn(fabsf(u[c]), gs.s), k, L);
+  }
+  float cf[4];
+  const float bias = (float)L;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float sign1 = __uint_as_float((__float_as_uint(u[c]) & 0x80000000u) | 0x3f800000u);   // +-1 with u's sign
+    e_next[c] = __fsub_rn(u[c], __fmaf_rn(idx[c], __fmul_rn(sign1, gs.half), 0.0f));
+    cf[c] = __fmaf_rn(idx[c], sign1, bias);
+  }
+  // two codes at a time (at most 16 bits), exact
+  const float up = exp2i(bits);
+  const unsigned lo = __float_as_uint(__fadd_rn(__fmaf_rn(cf[1], up, cf[0]), 8388608.0f)) & 0xffffu;
+  const unsigned hi = __float_as_uint(__fadd_rn(__fmaf_rn(cf[3], up, cf[2]), 8388608.0f)) & 0xffffu;
+  return lo | (hi << (2 * bits));
+}
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, "Parallel random numbers: as easy as 1, 2, 3",
 // SC 2011), from its published definition: ten rounds over a counter of four 32-bit words
 // under a key of two; a round multiplies words 0 and 2 by fixed odd constants, keeps both
@@ -496,6 +539,17 @@ __device__ __forceinline__ void pack_row_store_rt(int bits, unsigned c0, unsigne
     case 14: pack_row_store<14>(c0, c1, c2, c3, row_dst, lane); break;
     case 15: pack_row_store<15>(c0, c1, c2, c3, row_dst, lane); break;
     default: pack_row_store<16>(c0, c1, c2, c3, row_dst, lane); break;
+  }
+}
+
+// A lane's four codes already gathered into one field of 4 * bits bits, 4 <= bits <= 8.
+__device__ __forceinline__ void pack_row_store_fields_rt(int bits, unsigned field, void* row_dst, int lane) {
+  switch (bits) {
+    case 4: pack_row_store_fields<4>(field, row_dst, lane); break;
+    case 5: pack_row_store_fields<5>(field, row_dst, lane); break;
+    case 6: pack_row_store_fields<6>(field, row_dst, lane); break;
+    case 7: pack_row_store_fields<7>(field, row_dst, lane); break;
+    default: pack_row_store_fields<8>(field, row_dst, lane); break;
   }
 }
 

@@ -378,7 +378,8 @@ __device__ __forceinline__ void broadcast_row_ternary(const float xin[4], unsign
 // NW > 0: the worker count, known at compile time (the decode loop is unrolled and
 // every shared-memory offset is an immediate).  NW = 0: p.n workers, run-time loop.
 // GB: bits per gradient code, 2 (ternary) or 3 (five levels); 0: any grid with p.gbits
-// (3..8) bits per code, decoded through a table of the signed level values.
+// (3..8) bits per code, decoded through a table of the signed level values; 1: the uniform grid
+// with p.gbits (4..8) bits, whose level values are read off the codes by arithmetic.
 // XB: 2 when the weights are quantized to {-1/2, 0, 1/2} (kx = 0), which gets a path of its
 // own; 0: any p.kx, decided at run time.
 // ROWS: rows of 1024 elements per tile, 2 or 4 (a thread owns 4 elements of each row).
@@ -389,14 +390,14 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
                    const int inv_n_exact) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   PipeSmem* ps = reinterpret_cast<PipeSmem*>(smem_raw);
-  static_assert(GB == 0 || GB == 2 || GB == 3, "code widths of the pipelined decode");
+  static_assert(GB >= 0 && GB <= 3, "decodes of the pipelined pass");
   static_assert(XB == 0 || XB == 2, "weight code widths with a path of their own");
   static_assert(ROWS == 2 || ROWS == 4, "rows per tile");
   constexpr int kTile = ROWS * kPipeRowElems;
   unsigned char* stage_base = smem_raw + pipe_head_bytes(GB == 0);
   float* s_lut = reinterpret_cast<float*>(smem_raw + kPipeBarrierBytes);      // table decode only
   const int n = NW > 0 ? NW : p.n;
-  const int gb = GB > 0 ? GB : p.gbits;
+  const int gb = GB >= 2 ? GB : p.gbits;
   const unsigned stage_bytes = (unsigned)pipe_stage_bytes(n, SERVER_MOMENTS, gb, kTile);
   constexpr int kState = SERVER_MOMENTS ? 3 : 1;
   constexpr unsigned kCodesOff = kStageHeaderBytes + kState * kTile * 4;
@@ -490,9 +491,9 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
           bulk_load(sx + kTile, p.m + t.off, fbytes, &ps->full[s]);
           bulk_load(sx + 2 * kTile, p.v + t.off, fbytes, &ps->full[s]);
         }
-        // coordinate in words of the map: 32-bit (GB > 0) or 64-bit (table decode); the host
+        // coordinate in words of the map: 32-bit (GB >= 2) or 64-bit (the others); the host
         // only selects this kernel when the last tile's coordinate fits an int
-        const int c0 = GB > 0 ? (int)(t.off >> 5) * GB : (int)(t.off >> 6) * gb;
+        const int c0 = GB >= 2 ? (int)(t.off >> 5) * GB : (int)(t.off >> 6) * gb;
         tensor_load_2d(st + kCodesOff, &codes_map, c0, 0, &ps->full[s]);
       }
       ++issued;
@@ -530,13 +531,18 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
                             opaque_u32(144u << 23)};
     const FiveLevelLane fl = five_level_lane(lane);          // used by the 3-bit decode only
     // the 3-bit decode holds more per worker in registers: unroll it by 8 at most
-    constexpr int kUnroll = NW > 0 ? (GB == 0 && NW > 4 ? 4 : (GB == 3 && NW > 8 ? 8 : NW)) : 1;
+    constexpr int kUnroll = NW > 0 ? (GB < 2 && NW > 4 ? 4 : (GB == 3 && NW > 8 ? 8 : NW)) : 1;
     // table decode: the lane's 4 codes are the 4 * gb bits from bit 4 * gb * lane of the
     // warp's packed row (16 * gb bytes = 4 * gb words)
     const int tb_word = (4 * gb * lane) >> 5;
     const int tb_next = tb_word + 1 < 4 * gb ? tb_word + 1 : tb_word;
     const int tb_shift = (4 * gb * lane) & 31;
     const unsigned tb_cmask = (1u << gb) - 1u;
+    // uniform grid: codes 0 and 1 (2 and 3, once shifted down) of a field, moved into the mantissas of
+    // floats whose exponents give them the weight 1; less 2^E + L is the level index, times 2^-k the value
+    const unsigned un_m1 = tb_cmask << gb, un_g0 = 150u << 23, un_g1 = (unsigned)(150 - gb) << 23;
+    const float2 un_k = make_float2(-(exp2i(23) + (float)p.L), -(exp2i(23 - gb) + (float)p.L));
+    const float un_unit = GB == 1 ? exp2i(-p.k) : 0.0f;
 
     // Liveness vote.  With a max-abs scale most codes are level 0, and a worker whose 256
     // codes in this warp's two rows are all level 0 adds +0 to every sum, which changes
@@ -625,6 +631,13 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
             else       { r0.x = __fadd_rn(r0.x, v0); r1.x = __fadd_rn(r1.x, v1); }
           }
         };
+        auto uniform_accumulate = [&](float sc, unsigned f, float2& r0, float2& r1) {
+          const float2 unit = make_float2(un_unit, un_unit);
+          const float2 l0 = mul2_rn(level_pair(f, tb_cmask, un_g0, un_m1, un_g1, un_k), unit);          // exact
+          const float2 l1 = mul2_rn(level_pair(f >> (2 * gb), tb_cmask, un_g0, un_m1, un_g1, un_k), unit);
+          r0 = make_float2(__fadd_rn(r0.x, __fmul_rn(sc, l0.x)), __fadd_rn(r0.y, __fmul_rn(sc, l0.y)));
+          r1 = make_float2(__fadd_rn(r1.x, __fmul_rn(sc, l1.x)), __fadd_rn(r1.y, __fmul_rn(sc, l1.y)));
+        };
         auto row_pair = [&](int q) -> float2(&)[4] { return *reinterpret_cast<float2(*)[4]>(&a[4 * q]); };
         auto contribute = [&](int i) {
           const float2 sc = s_scale[i];
@@ -635,6 +648,9 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
                                 s_codes[i * kRunBytes + (2 * q + 1) * kRowBytes], k01, k23, mg, row_pair(q));
             } else if constexpr (GB == 3) {
               decode_accumulate5<false>(sc, window(i, 2 * q), window(i, 2 * q + 1), fl, row_pair(q));
+            } else if constexpr (GB == 1) {
+              uniform_accumulate(sc.x, field(i, 2 * q), a[4 * q], a[4 * q + 1]);
+              uniform_accumulate(sc.x, field(i, 2 * q + 1), a[4 * q + 2], a[4 * q + 3]);
             } else {
               table_accumulate(sc.x, field(i, 2 * q), field(i, 2 * q + 1), q);
             }
@@ -666,7 +682,7 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
 #pragma unroll
             for (int q = 0; q < ROWS / 2; ++q)
               decode_accumulate5<true>(s_scale[i], window(i, 2 * q), window(i, 2 * q + 1), fl, row_pair(q));
-        } else if constexpr (NW > 0 && GB > 0) {
+        } else if constexpr (NW > 0 && GB >= 2) {
           constexpr int kSlots = ROWS * vote_pieces_pow2(GB);      // v_slots, at compile time
           constexpr int kBallots = (NW * kSlots + 31) / 32;
           unsigned bal[kBallots];

@@ -559,6 +559,8 @@ worker_resident_kernel(const WorkerResidentParams rp) {
           code[0] = quantize_ternary4(uu, gs, en);             // the lane's byte of four codes
         } else if constexpr (MODE == G_FIVE) {
           code[0] = quantize_five4(uu, gs, en);                // the lane's 12 bits of four codes
+        } else if constexpr (MODE == G_UNIFORM) {
+          code[0] = quantize_uniform4(uu, gs, p.k, p.L, p.bits, en);
         } else {
 #pragma unroll
           for (int c = 0; c < 4; ++c) code[c] = quantize_grad<MODE>(uu[c], gs, p.k, p.L, en[c]);
@@ -570,6 +572,8 @@ worker_resident_kernel(const WorkerResidentParams rp) {
           store_row_of_code_bytes(code[0], dst, lane);
         } else if constexpr (MODE == G_FIVE) {
           pack_row_store_fields<3>(code[0], dst, lane);
+        } else if constexpr (MODE == G_UNIFORM) {
+          pack_row_store_fields_rt(p.bits, code[0], dst, lane);
         } else {
           pack_row_store_rt(p.bits, code[0], code[1], code[2], code[3], dst, lane);
         }

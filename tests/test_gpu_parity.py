@@ -820,3 +820,30 @@ def test_five_level_decision_around_both_midpoints_and_at_the_ends_of_the_fast_r
         assert np.array_equal(p.cpu.scales[:, 0], scales)
         assert bits_equal(p.gpu.e.cpu().numpy(), p.cpu.e), "e differs"
         p.close()
+
+
+@pytest.mark.parametrize("streaming", [True, False])
+@pytest.mark.parametrize("kg", [2, 3, 4, 5, 6])
+def test_uniform_decision_around_every_midpoint(kg, streaming):
+    # the index is the nearest integer of an estimate unless it lies near a half, where the division
+    # decides: coordinates a few ulps around every midpoint and around the ends of that band, of
+    # either sign, for scales at and beyond the ends of the range the estimate is used for
+    import paper_2004_14180_b200 as qb
+    c = np.arange(2 ** kg, dtype=np.float64)[:, None]
+    near = np.concatenate([np.arange(-4, 5) * 2.0 ** -23, [2.0 ** -14, -(2.0 ** -14), 2.0 ** -13, -(2.0 ** -13)]])
+    y = ((c + 0.5) / 2 ** kg * (1.0 + near / (c + 0.5))).ravel()
+    segs = []
+    for s in (1.37, 1.0, 3.3e-31, 1.1e-30, 2.9e38, 5e-44):
+        u = (np.concatenate([[1.0, -0.0, 0.0], y, -y]) * s).astype(np.float32)
+        u[0] = np.float32(s)
+        segs.append(u)
+    seg = [len(u) for u in segs]
+    opt = qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING) if streaming else None
+    p = Pair(seg, 2, kg, 0, S_MODE, x1=np.zeros(sum(seg), np.float32), grid_g=1, options=opt)
+    g = np.concatenate(segs)
+    gp = p.cpu.to_padded(np.stack([g, -g]))
+    p.gpu.worker_compress(1, torch.from_numpy(gp).cuda(), 0, 2, 1e-3)
+    p.cpu.workers_step(gp, 1e-3, 1)
+    p.compare_worker_outputs()
+    assert bits_equal(p.gpu.e.cpu().numpy(), p.cpu.e)
+    p.close()
