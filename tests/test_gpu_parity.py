@@ -847,3 +847,20 @@ def test_uniform_decision_around_every_midpoint(kg, streaming):
     p.compare_worker_outputs()
     assert bits_equal(p.gpu.e.cpu().numpy(), p.cpu.e)
     p.close()
+
+
+@pytest.mark.parametrize("kx", [1, 2, 6, 10, 14])
+def test_weight_decision_around_midpoints_and_clip(kx):
+    # Q_x takes a ceiling by a directed rounding: midpoints (ties toward zero) and their neighbours
+    # of either sign, grid points, zeros of either sign, subnormals, the clip at 1/2 and beyond
+    c = np.unique(np.linspace(0, 2 ** kx - 1, 200).astype(np.int64))
+    mids = ((c + 0.5) / 2 ** (kx + 1)).astype(np.float32)
+    x = np.concatenate([mids, np.nextafter(mids, np.float32(9)), np.nextafter(mids, np.float32(0)),
+                        (c / 2 ** (kx + 1)).astype(np.float32),
+                        np.array([0.0, 1e-45, 1e-39, 0.5, 0.50001, 3.0, 1e30], np.float32)])
+    x = np.concatenate([x, -x]).astype(np.float32)
+    p = Pair([x.size], 1, 0, kx, S_MODE, x1=x, want_wresid=True)
+    p.compare_state()                                  # the broadcast of x_1
+    p.step(np.zeros((1, x.size), np.float32))          # and the one of the server pass, x unchanged
+    p.compare_state()
+    p.close()
