@@ -655,7 +655,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
         (!c->geo.btiles.empty() &&
          !cuda_ok(cudaMemcpyAsync(c->d_btiles, c->geo.btiles.data(), c->geo.btiles.size() * sizeof(Tile),
                                   cudaMemcpyHostToDevice, c->stream))))) ||
-      // launches of the on-chip worker kernel count from 1, words of launch 0 are empty
+      // launches of the on-chip worker kernel count from 1, words of number 0 are empty
       (c->grid_resident > 0 && c->d_words != nullptr &&
        (!cuda_ok(cudaMemsetAsync(c->d_words, 0, c->geo.words_bytes, c->stream)) ||
         !cuda_ok(cudaMemsetAsync(c->d_epoch, 0, 2 * sizeof(unsigned), c->stream)) ||
@@ -768,6 +768,7 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
       WorkerResidentParams rp;
       rp.w = p;
       rp.words = use_words ? c->d_words : nullptr;
+      rp.num_words = use_words ? (long long)c->cfg.n * p.S * c->grid_resident : 0;
       rp.epoch = c->d_epoch;
       rp.rtiles = c->d_rtiles;
       rp.done = c->d_done;

@@ -76,7 +76,8 @@ struct WorkerResidentParams {
   unsigned* done;         // [n][S] tiles counted per pair, zeroed before the launch (as are the scales)
   unsigned long long* words;  // [n][S][gridDim.x] or nullptr: per (pair, CTA) {epoch : 24, tiles : 8, max |u| bits : 32};
                               // when given, it replaces `done` and the atomics
-  unsigned* epoch;            // {number of this launch (24 bits), CTAs that have left it}: a word of another launch
+  long long num_words;        // how many words there are
+  unsigned* epoch;            // {number of this launch (1 .. 2^24 - 1), CTAs that have left it}: a word of another launch
                               // does not count, so that nothing has to be cleared (the clears of the words, counters
                               // and scales were a quarter of the smallest steps: 18.8 -> 14 us)
   long long total;        // resident tiles of the call: its workers x TR
@@ -584,14 +585,26 @@ worker_resident_kernel(const WorkerResidentParams rp) {
   __syncthreads();
   if constexpr (WORDS) {
     // The last CTA to leave numbers the next launch: every CTA has read the number by then.  On the
-    // device, not in an argument, so that a captured launch can be replayed.  (A word is rewritten
-    // by every call that compresses its worker, far fewer than 2^24 launches after the last time.)
-    if (tid == 0) {
-      __threadfence();
-      if (atomicAdd(rp.epoch + 1, 1u) == (unsigned)ctas - 1u) {
-        rp.epoch[1] = 0u;
-        rp.epoch[0] = (__ldcg(rp.epoch) + 1u) & 0xffffffu;
+    // device, not in an argument, so that a captured launch can be replayed.  Which CTA writes a
+    // pair's word depends on the first worker of the call, so a word can outlive any number of
+    // launches that cut the workers otherwise; before the numbers start again the last CTA
+    // therefore clears all words (nobody reads them any more), and a number never comes back to one.
+    if (warp == 0) {
+      int clear = 0;
+      if (lane == 0) {
+        __threadfence();
+        if (atomicAdd(rp.epoch + 1, 1u) == (unsigned)ctas - 1u) {
+          const unsigned next = (__ldcg(rp.epoch) + 1u) & 0xffffffu;
+          rp.epoch[1] = 0u;
+          rp.epoch[0] = next != 0u ? next : 1u;
+          if (next == 0u) {
+            __threadfence();
+            clear = 1;
+          }
+        }
       }
+      if (__shfl_sync(0xffffffffu, clear, 0))
+        for (long long i = lane; i < rp.num_words; i += 32) rp.words[i] = 0ull;
     }
   }
 }

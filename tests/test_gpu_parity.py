@@ -365,6 +365,42 @@ def test_on_chip_worker_words_of_earlier_launches_do_not_count(placement):
 
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
+def test_on_chip_worker_words_are_cleared_before_launch_numbers_start_again(placement):
+    # a word written while all workers were compressed in one call lies where calls for some workers
+    # never write; it must not be there any more when its launch number could come again
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    seg = [sms * 4096 // 2 + 300, 5000, 70000]
+    n, d = 3, sum(seg)
+    rng = np.random.default_rng(330 + placement)
+    p = Pair(seg, n, 0, 0, placement, x1=(rng.standard_normal(d) * 0.2).astype(np.float32))
+
+    def step(**kw):
+        p.step(_rand_grads(rng, n, d, 0.01 * 0.3 ** p.step_no), **kw)
+        p.compare_state()
+
+    ws = p.gpu.workspace
+    i32, i64 = ws[:ws.numel() // 8 * 8].view(torch.int32), ws[:ws.numel() // 8 * 8].view(torch.int64)
+    number = torch.ones(i32.shape, dtype=torch.bool, device=ws.device)
+    for t in range(3):                                 # the next launch's number counts up from 2
+        step()
+        number &= i32 == t + 2
+    at = number.nonzero().flatten()
+    assert at.numel() == 1, "the launch number"
+    i32[at] = (1 << 24) - 2
+    torch.cuda.synchronize()
+    step()
+    written = ((i64 >> 40) & 0xffffff == (1 << 24) - 2).nonzero().flatten()
+    assert written.numel() > n                         # a pair of several tiles writes one word per CTA
+    step()                                             # the last number
+    assert int(i32[at]) == 1
+    assert not bool(i64[written].any()), "words of earlier launches are still there"
+    step(split_workers=True)
+    step()
+    assert int(i32[at]) == 4
+    p.close()
+
+
+@pytest.mark.parametrize("placement", [S_MODE, W_MODE])
 def test_streaming_launches_only(placement):
     # worker_kernel = STREAMING sends every pair through the two streaming launches, the
     # route that otherwise only pairs too large for the chip, partial worker ranges and some
