@@ -859,9 +859,9 @@ int launch_server(qadam_ctx* c, float alpha, long long tb, long long te, long lo
       const Tile* table = c->pipe_wide ? c->d_tiles + tb : c->d_ptiles + pb;
       const int np = (int)(c->pipe_wide ? te - tb : pe - pb);
       const int pgrid = std::min(c->sm_count, np);
-      // The launch may overlap the end of the workers' (see wait_for_previous_launch): its blocks
-      // start where theirs have left, and its set-up is off the path (13 290 elements, n = 4:
-      // 14.3 -> 12.3 us a step; 2^20, n = 4: 30.2 -> 28.4).
+      // The launch may overlap the end of the workers' on-chip launch (see wait_for_previous_launch):
+      // its blocks start where theirs have left, and its set-up is off the path (13 290 elements,
+      // n = 4: 14.3 -> 12.3 us a step; 2^20, n = 4: 30.2 -> 28.4).
       cudaLaunchAttribute attr = {};
       attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr.val.programmaticStreamSerializationAllowed = 1;

@@ -488,7 +488,6 @@ __device__ __forceinline__ void deferred_row(const WorkerParams& p, const float4
 template <int MODE, bool L2>
 __global__ void __launch_bounds__(kThreads, L2 ? 2 : 3)
 worker_deferred_kernel(const WorkerParams p) {
-  let_next_launch_start();
   static_assert(MODE == G_TERNARY || MODE == G_FIVE, "grids the sweep serves");
   constexpr int kBits = MODE == G_TERNARY ? 2 : 3;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -601,7 +600,6 @@ worker_deferred_kernel(const WorkerParams p) {
 template <bool U_IN_E, int MODE, bool L2 = false>
 __global__ void __launch_bounds__(kThreads, MODE == G_STOCHASTIC && !L2 ? 1 : 3)
 worker_quantize_kernel(const WorkerParams p) {
-  let_next_launch_start();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // Tiles per round of loads, then of arithmetic and stores.  (Two per round when only e is
   // read, to have as many loads in flight as the two-array form, was measured slower.)
