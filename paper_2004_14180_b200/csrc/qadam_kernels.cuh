@@ -482,7 +482,9 @@ __device__ __forceinline__ void deferred_row(const WorkerParams& p, const float4
 //   many  blocks take tiles as a full pass does, every warp its rows of the tile          (- / 0.50 ms)
 //   few   a warp takes 32 chunks (4 tiles) at a time, one byte of flags per lane, and handles
 //         their rows four at a time, so that it keeps as many loads in flight as with full tiles;
-//         the flags and descriptors of its next 32 are fetched meanwhile                 (1.4 / 0.57 ms)
+//         the flags and descriptors of its next 32 are fetched meanwhile                 (1.4 / 0.57 ms).
+//         Where 32 chunks each would leave warps without any, a warp takes 16, 8, ... 1 (7 x 10^6
+//         elements, n = 1, a third of the rows left: 28 -> 16 us)
 // (A tile per warp: 2.0 / 0.54 ms; lists of the flagged rows per block: 1.8 / 0.53; 32 chunks from
 // tiles 7 MB apart: 2.9 / 0.69.)
 template <int MODE, bool L2>
@@ -531,27 +533,31 @@ worker_deferred_kernel(const WorkerParams p) {
     }
     return;
   }
-  // this lane's chunk of a span: flags, tile
-  const unsigned step = gridDim.x * (kThreads / 32) * 4u;  // tiles between a warp's spans
-  const int sub = lane & (kTileChunks - 1);
-  unsigned t_next = (blockIdx.x * (kThreads / 32) + warp) * 4u + (unsigned)(lane / kTileChunks);
+  // a span: 32 consecutive chunks, one per lane, or fewer as long as some warp would have none
+  const unsigned warps = gridDim.x * (kThreads / 32), chunks = total * kTileChunks;   // below 2^32: 512 elements each
+  unsigned span = 32u;
+  while (span > 1u && chunks < span * warps) span >>= 1;
+  unsigned c_next = (blockIdx.x * (kThreads / 32) + warp) * span + (unsigned)lane;
   unsigned fl_next = 0, wl_next = 0;
   Tile tile_next = Tile{0, 0, 0};
+  bool more = false;                                      // this lane has a chunk in the span
   auto fetch = [&]() {
     fl_next = 0;
-    if (t_next < total) {
-      fl_next = p.deferred[(long long)t_next * kTileChunks + sub];
-      wl_next = t_next / tpw;
-      tile_next = p.tiles[t_next - wl_next * tpw];
+    more = (unsigned)lane < span && c_next < chunks;
+    if (more) {
+      const unsigned t = c_next / kTileChunks;
+      fl_next = p.deferred[c_next];
+      wl_next = t / tpw;
+      tile_next = p.tiles[t - wl_next * tpw];
     }
   };
   fetch();
-  while (__any_sync(0xffffffffu, t_next < total)) {
+  while (__any_sync(0xffffffffu, more)) {
     const unsigned fl = fl_next, wl = wl_next;
-    const long long elem = tile_next.off + sub * kChunkElems;
+    const long long elem = tile_next.off + (int)(c_next & (kTileChunks - 1)) * kChunkElems;
     unsigned sb = 0;                                      // asked for now, looked at after the first rows' loads
     if (fl != 0u) sb = p.scale_bits[(long long)(p.worker_begin + (int)wl) * p.S + tile_next.seg];
-    t_next += step;
+    c_next += warps * span;
     fetch();
     unsigned pending = __ballot_sync(0xffffffffu, fl != 0u);
     unsigned rows = 0;                                    // flagged rows left of the chunk of lane `cur`

@@ -423,7 +423,8 @@ def test_streaming_launches_only(placement):
 @pytest.mark.parametrize("l2", [0.0, 5e-4])
 def test_streaming_sweep_settles_rows_before_the_scale_is_known(kg, grid, l2):
     # Pairs too large for the chip (here: every pair, by option) are swept once; rows that a lower
-    # bound of the scale shows to be all level 0 are finished there, the others by a second kernel.
+    # bound of the scale shows to be all level 0 are finished there, the others by a second kernel
+    # (here nearly all; the grids with more than five levels take two full passes on the same inputs).
     # Lengths around the rows of 128, chunks of 512 and tiles of 4096 elements; the maximum at the
     # front, at the end and in the middle; coordinates exactly on the lowest midpoint and next to
     # it; zeros of either sign, a segment of zeros, one of subnormal magnitudes.
@@ -452,6 +453,60 @@ def test_streaming_sweep_settles_rows_before_the_scale_is_known(kg, grid, l2):
         g[:, off[8]:off[9]] = np.where(rng.random((n, seg[8])) < 0.5, np.float32(0.0), np.float32(-0.0))
         g[:, off[9]:off[10]] = (rng.integers(-7, 8, (n, seg[9])) * 1e-45).astype(np.float32)
         p.step(g, split_workers=t == 1)
+        p.compare_state()
+    p.close()
+
+
+def _gradients_of_few_open_rows(rng, seg, n, step):
+    """Small values, the pair's maximum once in every 512 elements (the stretch one warp of the sweep
+    settles), values of other levels in one row of 128 in thirty.  Returns the gradients and their rows'
+    largest magnitudes over the pair's."""
+    d = sum(seg)
+    g = (rng.standard_normal((n, d)) * 1e-3).astype(np.float32)
+    rows = []
+    for w in range(n):
+        big, a = np.float32(1 + 0.5 * w + 0.25 * step), 0
+        for length in seg:
+            v = g[w, a:a + length]
+            at = np.arange(0, length, 512)
+            v[at + rng.integers(0, np.minimum(512, length - at))] = big * rng.choice(np.float32([1, -1]), at.size)
+            at = np.arange(0, length, 128)
+            at = at[rng.random(at.size) < 1 / 30]
+            at = at + rng.integers(0, np.minimum(128, length - at))
+            keep = np.abs(v[at]) < big
+            v[at[keep]] = big * rng.choice(np.float32([0.4, -0.4, 0.8, -0.8]), int(keep.sum()))
+            full = np.zeros(-(-length // 128) * 128, np.float32)
+            full[:length] = np.abs(v)
+            rows.append(full.reshape(-1, 128).max(1) / big)
+            a += length
+    return g, np.concatenate(rows)
+
+
+@pytest.mark.parametrize("kg", [0, 1])
+@pytest.mark.parametrize("l2", [0.0, 5e-4])
+@pytest.mark.parametrize("chunks_per_warp", [0.2, 1.4, 2.7, 40])
+def test_rows_left_by_the_sweep_where_they_are_few(kg, l2, chunks_per_warp):
+    # The second kernel takes another way when fewer than half of the rows are left: spans of 1 to 32
+    # chunks of 512 elements per warp, by how many there are; one span per warp and several (the next
+    # span's flags are fetched ahead).  Every chunk holds the pair's maximum, so what the sweep
+    # leaves does not depend on the order in which it learns it: the rows with a value above the
+    # lowest midpoint.  Ragged tails, several segments, calls for some of the workers.
+    import paper_2004_14180_b200 as qb
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 3 * 8
+    n = 2
+    most = int(warps * chunks_per_warp) * 512 // n
+    seg = [most * 6 // 10 + 77, 130, 4096, most * 3 // 10 + 2000, 1, 513, most // 10 + 1]
+    d, tiles = sum(seg), n * sum(-(-length // 4096) for length in seg)
+    rng = np.random.default_rng(61 + kg)
+    p = Pair(seg, n, kg, 0, S_MODE, x1=(rng.standard_normal(d) * 0.2).astype(np.float32),
+             options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    p.set_regularization(l2)
+    for t in range(3 if chunks_per_warp < 10 else 1):
+        g, rows = _gradients_of_few_open_rows(rng, seg, n, t)
+        if t == 0:
+            left = int((rows > 0.5 ** (kg + 1)).sum())
+            assert 0 < left < 16 * tiles and left < 0.5 * rows.size
+        p.step(g, threads=8, split_workers=t == 1)
         p.compare_state()
     p.close()
 
