@@ -481,17 +481,22 @@ __device__ __forceinline__ void deferred_row(const WorkerParams& p, const float4
 // 10 % of the rows left; 1.4 x 10^8 Gaussian elements, n = 2, with nearly all of them left):
 //   many  blocks take tiles as a full pass does, every warp its rows of the tile          (- / 0.50 ms)
 //   few   a warp takes 32 chunks (4 tiles) at a time, one byte of flags per lane, and handles
-//         their rows four at a time, so that it keeps as many loads in flight as with full tiles;
+//         their rows four at a time (kBatch), so that it keeps as many loads in flight as with full tiles;
 //         the flags and descriptors of its next 32 are fetched meanwhile                 (1.4 / 0.57 ms).
 //         Where 32 chunks each would leave warps without any, a warp takes 16, 8, ... 1 (7 x 10^6
 //         elements, n = 1, a third of the rows left: 28 -> 16 us)
+// With the l2 term a warp of the second order takes two rows at a time, which fits three blocks on an
+// SM for either order; two blocks of 111 registers with four rows were slower than the two full
+// passes the sweep replaces where the rows are many (1.2 x 10^8 Gaussian elements, n = 2, lambda on,
+// this kernel: 0.63 -> 0.50 ms, with unquantized weights 0.84 -> 0.64; few: 0.21 / 0.22 ms).
 // (A tile per warp: 2.0 / 0.54 ms; lists of the flagged rows per block: 1.8 / 0.53; 32 chunks from
 // tiles 7 MB apart: 2.9 / 0.69.)
 template <int MODE, bool L2>
-__global__ void __launch_bounds__(kThreads, L2 ? 2 : 3)
+__global__ void __launch_bounds__(kThreads, 3)
 worker_deferred_kernel(const WorkerParams p) {
   static_assert(MODE == G_TERNARY || MODE == G_FIVE, "grids the sweep serves");
   constexpr int kBits = MODE == G_TERNARY ? 2 : 3;
+  constexpr int kBatch = L2 ? 2 : 4;                      // rows at a time where few are left
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned total = (unsigned)p.total_tiles, tpw = (unsigned)p.tiles_per_worker;
   const unsigned left = *p.deferred_rows;
@@ -563,11 +568,11 @@ worker_deferred_kernel(const WorkerParams p) {
     unsigned rows = 0;                                    // flagged rows left of the chunk of lane `cur`
     int cur = 0;
     while (pending | rows) {
-      long long row_elem[4];
-      int row_w[4], src[4];
-      bool have[4];
+      long long row_elem[kBatch];
+      int row_w[kBatch], src[kBatch];
+      bool have[kBatch];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
+      for (int a = 0; a < kBatch; ++a) {
         if (rows == 0u && pending != 0u) {
           cur = __ffs((int)pending) - 1;
           pending &= pending - 1u;
@@ -586,7 +591,7 @@ worker_deferred_kernel(const WorkerParams p) {
         if constexpr (L2) hw[a] = held_fetch(p, row_elem[a], lane);
       }
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
+      for (int a = 0; a < kBatch; ++a) {
         if (!have[a]) continue;
         const GradScale gs = grad_scale<MODE>(__uint_as_float(__shfl_sync(0xffffffffu, sb, src[a])), p.k);
         deferred_row<MODE, L2>(p, gv[a], ev[a], hw[L2 ? a : 0], gs, row_elem[a],
