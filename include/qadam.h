@@ -131,8 +131,10 @@ typedef struct {
  *  worker_kernel  AUTO: (worker, segment) pairs that fit in the SMs' shared memory go
  *                 through one persistent kernel that reads g and e once; larger pairs take
  *                 two streaming launches (max-abs, then quantize; or a sweep, then the rows it
- *                 left), and so do vectors of fewer than 2^20 elements under the stochastic
- *                 operator.  STREAMING: always the two launches.
+ *                 left), and so do, under the stochastic operator, vectors of fewer than 32
+ *                 segments with n * D below 2^23 (and D below 2^20 if the moments are on the
+ *                 workers).
+ *                 STREAMING: always the two launches.
  *  hand_over      how the persistent worker kernel passes a pair's scale between CTAs.
  *                 AUTO: one 64-bit word per (pair, CTA) while those fit in 32 MB of
  *                 workspace, else one counter per pair and atomics.  COUNTERS: always the

@@ -58,11 +58,6 @@ int grad_levels(int kg, int grid) {
 constexpr int kWordCtas = 256;                       // CTAs the per-pair words are sized for
 constexpr size_t kWordBudget = (size_t)32 << 20;     // bytes of workspace they may take
 
-// Elements from which the stochastic operator runs on chip: one pass over g, e against two
-// (ResNet-shaped, n = 8: 405 -> 255 us; 4.0 x 10^6 elements, n = 8: 152 -> 103).  Below it both
-// are a few microseconds of latency, and the streaming launches need no cooperative launch.
-constexpr int64_t kStochasticOnChip = 1 << 20;
-
 struct Geometry {
   std::vector<int64_t> seg_len, seg_off;
   int64_t D = 0;
@@ -128,6 +123,19 @@ int validate_config(const qadam_config* c) {
 // depends on the coin.
 bool sweeps(const qadam_config* c, GMode gmode) {
   return c->placement == QADAM_PLACE_SERVER && (gmode == G_TERNARY || gmode == G_FIVE);
+}
+
+// The stochastic operator on chip, or in two streaming launches.  On chip g and e are read once, but
+// every pair waits for a hand-over between the CTAs, which other pairs or a CTA's next tiles have to
+// cover.  Steps, streaming / on chip (time over time), one segment or eight, moments on the server:
+// n D = 2 x 10^6 0.86 .. 0.95, 4 .. 5 x 10^6 0.92 .. 0.98, 8.4 x 10^6 1.01 .. 1.13, 3.2 x 10^7 1.25 .. 1.32
+// (141 us / 108 at n = 32).  On the workers 8.4 x 10^6 is 1.09 .. 1.10, 3.2 x 10^7 1.30 .. 1.36 (227 us /
+// 169 at n = 32); below that 0.93 .. 1.09 with vectors of 2^20 elements (1.05 in the mean), 0.91 .. 1.17
+// with shorter ones.  64 segments: 0.99 .. 1.4 for either placement from n D = 2 x 10^4 on (33 us / 29
+// at n = 4, 10^6 elements, 200 segments).
+bool stochastic_on_chip(const qadam_config* c, int64_t D) {
+  return c->num_segments >= 32 || c->n * D >= (int64_t)1 << 23 ||
+         (c->placement == QADAM_PLACE_WORKER && D >= (int64_t)1 << 20);
 }
 
 int build_geometry(const qadam_config* c, Geometry* g) {
@@ -600,9 +608,8 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     int coop = 0, max_smem = 0;
     const bool want_split = o.worker_kernel == QADAM_WORKER_STREAMING;
     const bool wm = cfg->placement == QADAM_PLACE_WORKER;
-    // the stochastic operator in short vectors stays with the two streaming launches: see kStochasticOnChip
     const bool eligible = !want_split && c->geo.gmode != G_IDENTITY &&
-        (c->geo.gmode != G_STOCHASTIC || c->geo.D >= kStochasticOnChip) &&
+        (c->geo.gmode != G_STOCHASTIC || stochastic_on_chip(cfg, c->geo.D)) &&
         cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) && coop &&
         cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     if (eligible) {

@@ -756,6 +756,24 @@ def test_stochastic_ternary_operator_on_chip(placement):
     p.close()
 
 
+@pytest.mark.parametrize("placement", [S_MODE, W_MODE])
+@pytest.mark.parametrize("seg,n,on_chip", [([300] * 31, 2, (False, False)), ([300] * 32, 2, (True, True)),
+                                           ([1 << 16, 5000, 129], 3, (False, False)),
+                                           ([(1 << 20) - 256, 128], 7, (False, False)),
+                                           ([1 << 18] * 4, 7, (False, True)), ([1 << 18] * 4, 8, (True, True))])
+def test_stochastic_ternary_operator_at_the_ends_of_its_routes(placement, seg, n, on_chip):
+    # on chip from 32 segments or n * D = 2^23 on, with the moments on the workers also from D = 2^20 on
+    d = sum(seg)
+    rng = np.random.default_rng(930 + placement)
+    p = Pair(seg, n, 0, 1, placement, x1=(rng.standard_normal(d) * 0.2).astype(np.float32), grid_g=2, seed=78)
+    assert (p.gpu.worker_pass_model()[0] > 0) == on_chip[placement]
+    for t, lam in enumerate((0.0, 5e-4)):
+        p.set_regularization(lam)
+        p.step(_rand_grads(rng, n, d), threads=8, split_workers=t == 1)
+        p.compare_state()
+    p.close()
+
+
 def test_stochastic_operator_is_ternary_only():
     import paper_2004_14180_b200 as qb
     with pytest.raises(qb.QAdamError) as ei:
