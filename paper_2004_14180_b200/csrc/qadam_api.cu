@@ -563,10 +563,10 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
       delete c; return QADAM_ERR_CUDA;
     }
     const bool sm_mom = cfg->placement == QADAM_PLACE_SERVER;
-    const bool table = c->geo.gmode == G_POW2 || c->geo.gmode == G_UNIFORM;
+    const bool wide_words = c->geo.gmode == G_POW2 || c->geo.gmode == G_UNIFORM;
     const bool pipe_codes = c->geo.gmode == G_TERNARY || c->geo.gmode == G_STOCHASTIC || c->geo.gmode == G_FIVE ||
-                            (table && c->geo.gbits <= 8);
-    const size_t head = pipe_head_bytes(table);
+                            (wide_words && c->geo.gbits <= 8);
+    const size_t head = pipe_head_bytes(c->geo.gmode == G_POW2);
     const bool want_plain = o.server_kernel == QADAM_SERVER_PLAIN;
     auto stages_for = [&](int tile_elems) {
       const size_t sb = pipe_stage_bytes(cfg->n, sm_mom, pipe_codes ? c->geo.gbits : 2, tile_elems);
@@ -581,11 +581,11 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     const size_t sb = pipe_stage_bytes(cfg->n, sm_mom, pipe_codes ? c->geo.gbits : 2, tile_elems);
     int stages = stages_for(tile_elems);
     // the tensor copy addresses a tile's codes by a 32-bit coordinate in words of the stream
-    // (32-bit words, 64-bit for the table decode): longer streams take the plain kernel
-    const bool coord_fits = (long long)c->geo.gcode_bytes / (table ? 8 : 4) < (1ll << 31);
+    // (32-bit words, 64-bit for the geometric and uniform grids): longer streams take the plain kernel
+    const bool coord_fits = (long long)c->geo.gcode_bytes / (wide_words ? 8 : 4) < (1ll << 31);
     if (!want_plain && pipe_codes && coord_fits && cfg->n <= kPipeMaxWorkers && stages >= 2 &&
         make_codes_tensor_map(&c->codes_map, b->gcodes, (long long)c->geo.gcode_bytes, cfg->n,
-                              c->geo.gbits, table, tile_elems)) {
+                              c->geo.gbits, wide_words, tile_elems)) {
       c->pipe_stages = stages;
       c->pipe_smem = head + (size_t)stages * sb;
       if (!cuda_ok(cudaFuncSetAttribute(pick_pipe(c), cudaFuncAttributeMaxDynamicSharedMemorySize,

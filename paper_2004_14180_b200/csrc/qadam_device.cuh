@@ -71,11 +71,7 @@ __device__ __forceinline__ float adam_step(const Hyper& h, float m, float v, flo
 // comparison is then false and the index is 0.
 template <int MODE>
 __device__ __forceinline__ int level_index(float y, int k, int L) {
-  if constexpr (MODE == G_TERNARY) {
-    return y > 0.5f ? 1 : 0;
-  } else if constexpr (MODE == G_FIVE) {
-    return (y > 0.25f ? 1 : 0) + (y > 0.75f ? 1 : 0);
-  } else if constexpr (MODE == G_POW2) {
+  if constexpr (MODE == G_POW2) {
     // levels 0, 2^-k, 2^(1-k), ..., 1: midpoints 2^(-k-1), then 3*2^(c-3-k), c = 2..L
     float t = exp2i(-k - 1);
     int c = y > t ? 1 : 0;
@@ -99,9 +95,7 @@ __device__ __forceinline__ int level_index(float y, int k, int L) {
 // Magnitude of level c of G (exactly representable).
 template <int MODE>
 __device__ __forceinline__ float level_value(int c, int k) {
-  if constexpr (MODE == G_TERNARY) {
-    return c ? 1.0f : 0.0f;
-  } else if constexpr (MODE == G_FIVE) {
+  if constexpr (MODE == G_FIVE) {
     return 0.5f * (float)c;
   } else if constexpr (MODE == G_POW2) {
     return c ? exp2i(c - 1 - k) : 0.0f;
@@ -149,33 +143,17 @@ __device__ __forceinline__ GradScale grad_scale(float s, int k) {
 // s = |u|_inf, returns the code (level index + L) and writes e' = u - Q_g(u).
 template <int MODE>
 __device__ __forceinline__ unsigned quantize_grad(float u, const GradScale& gs, int k, int L, float& e_next) {
+  static_assert(MODE == G_POW2 || MODE == G_UNIFORM, "the other grids are quantized four coordinates at a time");
   const float s = gs.s;
   const float a = fabsf(u);
   const bool neg = u < 0.0f;
-  if constexpr (MODE == G_TERNARY) {
-    // The decision is y = fl(|u| / s) > 1/2.  |u| <= s/2 gives a quotient <= 1/2 (s/2 is exact
-    // for a normal s), and |u| > (s/2)(1 + 2^-21) gives a quotient whose rounding stays above
-    // 1/2.  Only values inside that band, and tiny or non-finite scales, take the division.
-    bool one;
-    if (a <= gs.half && gs.fast) {
-      one = false;
-    } else if (a > gs.half_hi && gs.fast) {
-      one = true;
-    } else {
-      one = __fdiv_rn(a, s) > 0.5f;
-    }
-    const float deq = one ? (neg ? -s : s) : 0.0f;
-    e_next = __fsub_rn(u, deq);
-    return one ? (neg ? 0u : 2u) : 1u;
-  }
   int c;
   bool decided = false;
-  if constexpr (MODE == G_FIVE || MODE == G_POW2) {
+  if constexpr (MODE == G_POW2) {
     // Geometric levels 0, 2^-k, ..., 1: the midpoints are 2^(-k-1) and 1.5 * 2^j, so the level
     // index is read off the exponent of y and of whether its fraction reaches 1.5.
     // y' = fl(|u| * fl(1/s)) is within 2^-22 (relative) of y; unless y' lies within 2^-19 of a
     // midpoint (fraction near 1 or near 1.5) both give the same index.
-    const int kk = MODE == G_FIVE ? 1 : k;
     if (gs.fast) {
       const float yp = __fmul_rn(a, gs.inv);
       const unsigned yb = __float_as_uint(yp);
@@ -183,23 +161,9 @@ __device__ __forceinline__ unsigned quantize_grad(float u, const GradScale& gs, 
       const bool near = (m - 0x3ffff0u) <= 0x20u || m <= 0x10u || m >= 0x7fffefu;
       if (!near) {
         const int e15 = (int)((yb + 0x00400000u) >> 23) - 127;      // exponent, plus one when the fraction is >= 1.5
-        const int upper = e15 + kk;
-        c = (yp > exp2i(-kk - 1) ? 1 : 0) + (upper > 0 ? upper : 0);
+        const int upper = e15 + k;
+        c = (yp > exp2i(-k - 1) ? 1 : 0) + (upper > 0 ? upper : 0);
         c = c > L ? L : c;
-        decided = true;
-      }
-    }
-  } else if constexpr (MODE == G_UNIFORM) {
-    // Uniform levels c / 2^k: the index is ceil(z - 1/2) with z = y 2^k.  z' = |u| * fl(2^k / s)
-    // is within 2^-22 (relative) of z; unless z' - 1/2 lies within 2^-15 of an integer (z <= 64)
-    // both give the same index.
-    if (gs.fast) {
-      const float t = __fadd_rn(__fmul_rn(a, gs.inv), -0.5f);
-      const float ct = ceilf(t);
-      const float w = __fsub_rn(ct, t);                              // in [0, 1)
-      if (w > 6.1035156e-05f && w < 0.99993896f) {
-        c = (int)ct;
-        c = c < 0 ? 0 : (c > L ? L : c);
         decided = true;
       }
     }
@@ -236,10 +200,10 @@ __device__ __forceinline__ float positive_as_one(float d) {
 }
 
 // Ternary Q_g of 4 consecutive coordinates of one lane, the error update, and the lane's byte of
-// packed codes (code = level index + 1, coordinate c in bits 2c, 2c + 1).  Same decisions as
-// quantize_grad<G_TERNARY>: level 1 iff fl(|u| / s) > 1/2, settled without dividing outside the
-// sliver (s/2, (s/2)(1 + 2^-21)], by the division inside it and for scales that are not ordinary
-// numbers.  Outside the sliver everything runs on the fp32 pipe (the integer pipe, at half its
+// packed codes (code = level index + 1, coordinate c in bits 2c, 2c + 1).  Level 1 iff fl(|u| / s) >
+// 1/2, settled without dividing outside the sliver (s/2, (s/2)(1 + 2^-21)]: |u| <= s/2 gives a
+// quotient <= 1/2 (s/2 is exact for a normal s), |u| > (s/2)(1 + 2^-21) one whose rounding stays above
+// 1/2.  The division decides inside it and for scales that are not ordinary numbers.  Outside the sliver everything runs on the fp32 pipe (the integer pipe, at half its
 // rate, is what the quantize kernels are otherwise bound by): [|u| > t] is sat((|u| - t) 2^127),
 // exact because the difference of two nearby floats is exact and at least 2^-125 for the scales
 // that take this path; the codes are gathered by exact multiply-adds and read out of a mantissa.
@@ -277,8 +241,8 @@ __device__ __forceinline__ unsigned quantize_ternary4(const float (&u)[4], const
 
 // Five-level Q_g (levels 0, 1/2, 1 times the scale, k_g = 1 of the geometric grid) of 4
 // consecutive coordinates of one lane, the error update, and the lane's 12 bits of packed codes
-// (code = level index + 2, coordinate c in bits 3c .. 3c + 2).  Same decisions as
-// quantize_grad<G_FIVE>: index [y > 1/4] + [y > 3/4] with y = fl(|u| / s).  y' = fl(|u| fl(1/s)) is
+// (code = level index + 2, coordinate c in bits 3c .. 3c + 2).  The index is
+// [y > 1/4] + [y > 3/4] with y = fl(|u| / s).  y' = fl(|u| fl(1/s)) is
 // within 2^-22 (relative) of y, so y' above t (1 + 2^-20) or at most t (1 - 2^-20) settles the
 // comparison with the midpoint t; a y' in between sends the lane's four coordinates to the
 // division.  As in quantize_ternary4 the comparisons are saturated differences on the fp32 pipe
@@ -326,7 +290,7 @@ __device__ __forceinline__ unsigned quantize_five4(const float (&u)[4], const Gr
 
 // Uniform Q_g (levels c / 2^k) of 4 consecutive coordinates of one lane, the error update, and the
 // lane's 4 * bits bits of packed codes (bits = k + 2, at most 8).  Same decisions as
-// quantize_grad<G_UNIFORM>: z' = |u| fl(2^k / s) is within 2^-16 of z = y 2^k, so its nearest integer
+// level_index<G_UNIFORM> of the quotient: z' = |u| fl(2^k / s) is within 2^-16 of z = y 2^k, so its nearest integer
 // (by adding and subtracting 1.5 2^23) is the index unless z' lies within 2^-14 of a half, where the
 // division decides for the lane's four coordinates.  On the fp32 pipe like the two above; the
 // dequantized value fl(index s / 2^k) is a multiply-add of +0, so that level 0 gives +0.

@@ -606,7 +606,9 @@ worker_deferred_kernel(const WorkerParams p) {
 // Worker phase 2: codes = Q_g level indices of u against the finished scale,
 // packed; e <- u - Q_g(u).  U_IN_E: u was left in e's slot by phase 1.
 // Three blocks per SM (at most 80 registers): with one block of 150 registers the
-// general grids ran at 0.35 of the copy rate, with three at 0.73 (measured).
+// general grids ran at 0.35 of the copy rate, with three at 0.73 (measured).  The stochastic
+// operator's kernels keep to 80 registers by themselves and lose by the bound (3 x 10^7 elements,
+// n = 4, a step: 543 us without, 564 with it; 813 and 831 with the moments on the workers).
 // ---------------------------------------------------------------------------
 template <bool U_IN_E, int MODE, bool L2 = false>
 __global__ void __launch_bounds__(kThreads, MODE == G_STOCHASTIC && !L2 ? 1 : 3)

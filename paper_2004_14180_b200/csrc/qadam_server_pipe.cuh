@@ -378,7 +378,7 @@ __device__ __forceinline__ void broadcast_row_ternary(const float xin[4], unsign
 
 // NW > 0: the worker count, known at compile time (the decode loop is unrolled and
 // every shared-memory offset is an immediate).  NW = 0: p.n workers, run-time loop.
-// GB: bits per gradient code, 2 (ternary) or 3 (five levels); 0: any grid with p.gbits
+// GB: bits per gradient code, 2 (ternary) or 3 (five levels); 0: the geometric grid with p.gbits
 // (3..8) bits per code, decoded through a table of the signed level values; 1: the uniform grid
 // with p.gbits (4..8) bits, whose level values are read off the codes by arithmetic.
 // XB: 2 when the weights are quantized to {-1/2, 0, 1/2} (kx = 0), which gets a path of its
@@ -415,9 +415,7 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
       const int q = c - p.L;
       const int a = q < 0 ? -q : q;
       float lv = 0.0f;
-      if (a != 0 && a <= p.L)
-        lv = p.gmode == G_POW2 ? level_value<G_POW2>(a, p.k)
-                               : (p.gmode == G_FIVE ? level_value<G_FIVE>(a, p.k) : level_value<G_UNIFORM>(a, p.k));
+      if (a != 0 && a <= p.L) lv = level_value<G_POW2>(a, p.k);
       s_lut[c] = q < 0 ? -lv : lv;
     }
   }
@@ -540,7 +538,7 @@ server_pipe_kernel(const ServerParams p, const __grid_constant__ CUtensorMap cod
                             opaque_u32(144u << 23)};
     const FiveLevelLane fl = five_level_lane(lane);          // used by the 3-bit decode only
     // the 3-bit decode holds more per worker in registers: unroll it by 8 at most
-    constexpr int kUnroll = NW > 0 ? (GB < 2 && NW > 4 ? 4 : (GB == 3 && NW > 8 ? 8 : NW)) : 1;
+    constexpr int kUnroll = NW > 0 ? (GB == 3 && NW > 8 ? 8 : NW) : 1;
     // table decode: the lane's 4 codes are the 4 * gb bits from bit 4 * gb * lane of the
     // warp's packed row (16 * gb bytes = 4 * gb words)
     const int tb_word = (4 * gb * lane) >> 5;
