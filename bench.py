@@ -176,9 +176,9 @@ def algorithmic_bytes(kernel: str, w, placement: str, D: int, gbits: int, xbits:
     """Bytes one launch of `kernel` must move at its interface (fp32 state it has
     to read and write, packed codes), for all n workers.  The worker side is capacity
     aware: (worker, segment) pairs that fit on chip go through the fused kernel and are
-    counted once (one pass); larger ones take the two streaming launches: a sweep that settles
-    most of them, or two passes (the max-abs scale needs the whole pair before any of it can be
-    quantized)."""
+    counted once (one pass); larger ones take the two streaming launches: a sweep and the rows it
+    leaves ("sweep", both launches together), or two passes (the max-abs scale needs the whole pair
+    before any of it can be quantized)."""
     n = w.n
     server_moments = placement == "server"
     # with the l2 term a worker also reads the weights it holds: the packed broadcast, or x
@@ -189,11 +189,11 @@ def algorithmic_bytes(kernel: str, w, placement: str, D: int, gbits: int, xbits:
         return one_pass * ((12.0 if server_moments else 28.0) + held + gbits / 8.0)
     # the split launches cover everything, or, beside the fused kernel, the two-pass pairs only
     split_units = pass_model[1] if pass_model and pass_model[0] > 0 else n * D
-    # ternary and five-level codes, moments on the server: the sweep settles every row it can in one
-    # pass, and what its second kernel reads again (rows whose codes are not all level 0, which
-    # depends on the data) is not counted
-    if server_moments and w.kg in (0, 1) and kernel in ("absmax", "quantize"):
-        return (12.0 + held + gbits / 8.0) * split_units if kernel == "absmax" else 0.0
+    # ternary and five-level codes, moments on the server: the sweep writes e and the codes of the rows
+    # it settles, the second kernel of the others (how many depends on the data); together every
+    # array is touched once, and the rows left are read again, which is not counted
+    if kernel == "sweep":
+        return (12.0 + held + gbits / 8.0) * split_units
     if kernel == "absmax":      # phase 1: read g, e (worker moments: + read m, v, write m, v, u)
         per = (8.0 if server_moments else 28.0) + held
         return per * split_units
@@ -323,10 +323,18 @@ def alu_decode_peak():
 
 
 def kernel_table(prof, w, placement_name, q, weight_decay, peak, weight_feedback=False):
-    """Per kernel: launches, time, algorithmic bytes, achieved rate and its fractions."""
+    """Per kernel: launches, time, algorithmic bytes, achieved rate and its fractions.  The sweep
+    and the kernel for the rows it leaves share out one pass between them by the data: they are one
+    entry, a launch of it being one of each."""
     D = q.D
     kernels = {}
+    prof = dict(prof)
     total_ms = sum(m for m, c in prof.values()) or 1.0
+    parts = None
+    if placement_name == "server" and w.kg in (0, 1) and prof["absmax"][1] and prof["quantize"][1]:
+        (ms_s, cnt), (ms_r, _) = prof.pop("absmax"), prof.pop("quantize")
+        prof = {"sweep": (ms_s + ms_r, cnt), **prof}
+        parts = [ms_s / cnt, ms_r / cnt]
     for name, (ms, cnt) in prof.items():
         if cnt == 0:
             continue
@@ -338,6 +346,8 @@ def kernel_table(prof, w, placement_name, q, weight_decay, peak, weight_feedback
         kernels[name] = {"launches": int(cnt), "ms_per_launch": per, "share": ms / total_ms,
                          "algorithmic_bytes": bytes_, "achieved_gbs": gbs,
                          "frac": gbs / peak, "frac_of_nominal": gbs / NOMINAL_HBM_GBS}
+        if name == "sweep":
+            kernels[name]["ms_sweep_and_rows_left"] = parts
         if name == "server" and w.kg == 0:
             # second roofline of the server pass: with dense codes (always, when the moments are on
             # the workers) it is bound by the arithmetic of the decode, not by HBM
@@ -462,6 +472,8 @@ def config_records(args, dev, world, peak):
                     "kernels": {k: {"ms_per_launch": v["ms_per_launch"], "launches": v["launches"],
                                     "achieved_gbs": v["achieved_gbs"], "frac": v["frac"],
                                     "frac_of_nominal": v["frac_of_nominal"],
+                                    **({"ms_sweep_and_rows_left": v["ms_sweep_and_rows_left"]}
+                                       if "ms_sweep_and_rows_left" in v else {}),
                                     **({"alu_frac": v["alu"]["frac"]} if "alu" in v else {})}
                                 for k, v in m.kernels.items()}})
         m.close()
@@ -521,15 +533,14 @@ def run_b200(args):
     # ---- roofline of the dominant kernel ---------------------------------------------
     dom = max(kernels, key=lambda k: kernels[k]["launches"] * kernels[k]["ms_per_launch"])
     traffic, traffic_note = None, None
-    tkey = f"{dom}:{args.placement}"
-    trec = ncu_traffic().get(tkey)
-    if trec and args.weight_decay == 0.0:
-        if trec.get("digest") == csrc_digest():
+    table = ncu_traffic()
+    trec = [table.get(f"{k}:{args.placement}") for k in (("absmax", "quantize") if dom == "sweep" else (dom,))]
+    if all(trec) and args.weight_decay == 0.0:
+        if all(r.get("digest") == csrc_digest() for r in trec):
             one_pass, two_pass = q.worker_pass_model()
-            units = {"worker_fused": one_pass, "absmax": two_pass if one_pass else w.n * D,
-                     "quantize": two_pass if one_pass else w.n * D}.get(dom, D)
-            traffic = trec["bytes_per_unit"] * units
-            traffic_note = trec.get("case")
+            units = {"worker_fused": one_pass, "sweep": two_pass, "absmax": two_pass, "quantize": two_pass}.get(dom, D)
+            traffic = sum(r["bytes_per_unit"] for r in trec) * units
+            traffic_note = trec[0].get("case")
         else:
             traffic_note = "the kernel sources changed since the counters were taken"
     roofline = {"bound": "hbm", "kernel": dom, "achieved": kernels[dom]["achieved_gbs"],
