@@ -209,7 +209,8 @@ int build_geometry(const qadam_config* c, Geometry* g) {
     g->off_epoch = wo;
     wo += 256;
   }
-  // flags of the rows the sweep leaves to the second kernel (1 / 8192 of the size of e)
+  // flags of the rows the sweep leaves to the second kernel: a byte per 512 elements, 8 per tile
+  // however short (1 / 2048 of the size of e where tiles are full)
   g->off_deferred = wo;
   if (sweeps(c, g->gmode))
     wo += 256 + (size_t)round_up64((int64_t)c->n * (int64_t)g->tiles.size() * kTileChunks, 256);   // a count first
@@ -233,7 +234,7 @@ struct qadam_ctx {
   int64_t launches;
   int grid_absmax, grid_quant, grid_ident, grid_server, grid_bcast;
   size_t server_smem;
-  // persistent pipelined server pass (ternary codes): stages > 0 when in use
+  // persistent pipelined server pass: stages > 0 when in use
   float lambda = 0.0f;       // l2 term (qadam_set_regularization)
   int pipe_stages = 0;
   size_t pipe_smem = 0;
@@ -555,7 +556,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
       !cuda_ok(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->server_smem))) {
     delete c; return QADAM_ERR_CUDA;
   }
-  // The pipelined server pass needs ternary or five-level codes, at most kPipeMaxWorkers streams and room
+  // The pipelined server pass needs codes of at most 8 bits, at most kPipeMaxWorkers streams and room
   // for at least two stages in shared memory; otherwise the plain grid-stride kernel runs.
   {
     int max_smem = 0;
@@ -629,8 +630,8 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
         c->res_slots = slots;
         c->res_estages = estages;
         c->res_smem = resident_smem_bytes(slots, estages, wm, 0);
-        // with the l2 term one slot less (two for unquantized weights): still as many as the largest
-        // pair gives a CTA, so the loads of a pair never wait for its own stores
+        // with the l2 term up to two slots less: still at least as many as the largest pair gives a
+        // CTA, so the loads of a pair never wait for its own stores
         c->res_slots_l2 = slots_for(held);
         c->res_smem_l2 = resident_smem_bytes(c->res_slots_l2, estages, wm, held);
         bool fits = !c->geo.rtiles.empty() && c->res_slots_l2 >= slots - spare;

@@ -9,7 +9,8 @@
 // to memory for the second look costs as much through L2 as from HBM on this machine
 // (the path from L2 into an SM carries little more than HBM delivers: measured), so the
 // only way to touch each element once is to hold u where it was computed.  Each of the
-// 148 SMs keeps a ring of 12 slots of 4096 values (8 when m and v are staged too); a pair
+// 148 SMs keeps a ring of 12 slots of 4096 values (8 when m and v are staged too, one or two
+// fewer with the l2 term); a pair
 // spread over all SMs may therefore be up to a few million elements long.  Per pair and
 // element this moves g, e in and e', the packed code out: 12 + b_g / 8 bytes (28 + b_g / 8
 // with m, v read and written), the least the method allows.
@@ -34,8 +35,9 @@
 // scale that fits one tile) skips the global record: the dispatcher takes the maximum
 // from the tile's header in shared memory.  No deadlock: a load waits for the store of the tile `slots`
 // places earlier in the same CTA, which waits for that tile's pair to be complete, which
-// waits for loads of that pair only; a pair gives a CTA fewer tiles than it has slots
-// (the host sends larger pairs elsewhere), so those loads wait, in turn, only for
+// waits for loads of that pair only; a pair gives a CTA at most as many tiles as it has slots
+// (the host sends larger pairs elsewhere; with the l2 term it can be just as many), so none of
+// its loads needs the slot of another of its tiles: they wait, in turn, only for
 // stores of OLDER pairs, and the oldest unfinished pair can always finish, provided
 // every CTA is resident (cooperative launch).  All waits are bounded: when one runs out
 // the TIMEOUT bit of the status word is set and every role leaves its loop.
@@ -73,7 +75,7 @@ struct __align__(8) RTile {
 struct WorkerResidentParams {
   WorkerParams w;
   const RTile* rtiles;    // [TR]
-  unsigned* done;         // [n][S] tiles counted per pair, zeroed before the launch (as are the scales)
+  unsigned* done;         // [n][S] tiles counted per pair, zeroed before the launch (as are the scales) when it is used
   unsigned long long* words;  // [n][S][gridDim.x] or nullptr: per (pair, CTA) {epoch : 24, tiles : 8, max |u| bits : 32};
                               // when given, it replaces `done` and the atomics
   long long num_words;        // how many words there are
@@ -82,7 +84,7 @@ struct WorkerResidentParams {
                               // and scales were a quarter of the smallest steps: 18.8 -> 14 us)
   long long total;        // resident tiles of the call: its workers x TR
   int TR;                 // resident tiles per worker
-  int slots;              // slots of the CTA's ring (a pair gives a CTA fewer tiles than this)
+  int slots;              // slots of the CTA's ring (a pair gives a CTA at most this many tiles)
   int estages;            // stages of the e ring
   int held_bytes;         // l2 term: bytes of a tile's held weights, which a stage then carries too
 };
@@ -91,10 +93,9 @@ struct WorkerResidentParams {
 // moments on the server the load side only adds (8 warps, 4 rows of 1024 elements per
 // thread and tile) and the store side quantizes (16 warps, 2 rows); with the moments on
 // the workers the load side also runs the moment updates, a root and a division per
-// element (16 warps) and the store side gets 8; the same 16 / 8 split serves the l2 term,
-// whose decode of the held weights is load-side work.  The held weights of a tile come with
-// its stage (a bulk copy of the packed codes, or of x): read from global memory where they are
-// used, their latency was paid once per tile.
+// element (16 warps) and the store side gets 8.  The l2 term changes neither split: its held
+// weights come with the tile's stage (a bulk copy of the packed codes, or of x; read from global
+// memory where they are used, their latency was paid once per tile).
 constexpr int kRColThreads = 256;       // threads across a 1024-element row, 4 elements each
 constexpr int kRConsumerWarps = 24;
 constexpr int kRRoleWarp0 = kRConsumerWarps;      // producer, publisher, dispatcher follow

@@ -266,9 +266,8 @@ def test_on_chip_worker_capacity_boundary(placement):
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
 @pytest.mark.parametrize("kx", [0, 3, 6, 9, -1])
 def test_on_chip_worker_l2_term_many_tiles(kx, placement):
-    # the l2 term inside the on-chip kernel with several tiles per CTA: the held-weight
-    # codes of a tile are fetched while the tile before it is processed (widths up to 8
-    # bits); wider codes and unquantized weights are read in place
+    # the l2 term inside the on-chip kernel with several tiles per CTA: the held weights of a
+    # tile (packed codes of any width, or x itself) come with the tile's stage of the ring
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     seg = [sms * 3 * 4096 + 300, 5000, 70000, 129]
     n, d = 3, sum([sms * 3 * 4096 + 300, 5000, 70000, 129])
