@@ -14,7 +14,9 @@ an independent replica of the workload: the path has no exchange step between
 GPUs, so there is no collective in the data path; the time is the maximum over
 ranks and the value the elements all ranks processed per second.
 
-One JSON line is printed by rank 0.
+One JSON line is printed by rank 0, short enough (LINE_CHARS) to be read back from the end of a log: numbers
+of six digits, and the other configurations in brief under `configs` ("workload workers placement
+[decay] [feedback]: ms per step, fraction of the measured copy rate"); `--records FILE` has them in full.
 """
 from __future__ import annotations
 
@@ -33,6 +35,7 @@ if ROOT not in sys.path:
 
 METRIC = "qadam_ef_step_elements_per_s"
 UNIT = "elements/s"
+LINE_CHARS = 2900            # the printed line stays below this
 FALLBACK_HBM_GBS = 6650.0
 
 NOMINAL_HBM_GBS = 8000.0     # the B200's HBM3e figure the 75 % target is stated against
@@ -91,6 +94,7 @@ def parse_args():
                          "workers dealt out to the ranks and the server sharded (codes exchanged over NCCL)")
     ap.add_argument("--no-configs", action="store_true",
                     help="skip the per-configuration records (key `configs` of the line)")
+    ap.add_argument("--records", default=None, help="file for the full per-configuration records, a JSON line each")
     ap.add_argument("--config-steps", type=int, default=5)
     ap.add_argument("--sample-log2", type=int, default=None,
                     help="log2 of the per-worker sample length the oracle is timed on")
@@ -352,8 +356,7 @@ def kernel_table(prof, w, placement_name, q, weight_decay, peak, weight_feedback
             # second roofline of the server pass: with dense codes (always, when the moments are on
             # the workers) it is bound by the arithmetic of the decode, not by HBM
             codes = float(w.n) * D / (per * 1e-3)
-            kernels[name]["alu"] = {"bound": "alu", "achieved": codes, "peak": alu_decode_peak(),
-                                    "unit": "codes/s", "frac": codes / alu_decode_peak()}
+            kernels[name]["alu"] = {"codes_per_s": codes, "frac": codes / alu_decode_peak()}
     return kernels
 
 
@@ -483,6 +486,34 @@ def config_records(args, dev, world, peak):
     return out
 
 
+def six_digits(v):
+    """Floats cut to six significant digits, more than any timing here has."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: six_digits(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [six_digits(x) for x in v]
+    return v
+
+
+def printed_line(line):
+    """The line as it is printed; as many configurations from the end of the list as would make it
+    too long to be read back are left out."""
+    line = six_digits(line)
+    while len(json.dumps(line)) >= LINE_CHARS and line.get("configs"):
+        line["configs"].pop()
+    return json.dumps(line)
+
+
+def config_brief(rec):
+    what = f"{rec['workload']} {rec['n_workers']} {rec['placement'][0]}"
+    what += (" decay" if rec["weight_decay"] else "") + (" feedback" if rec["weight_feedback"] else "")
+    if "skipped" in rec:
+        return f"{what}: skipped"
+    return f"{what}: {rec['ms_per_step']:.4g}, {rec['step_frac']:.2f}"
+
+
 def run_b200(args):
     import torch
     import torch.distributed as dist
@@ -546,7 +577,7 @@ def run_b200(args):
     roofline = {"bound": "hbm", "kernel": dom, "achieved": kernels[dom]["achieved_gbs"],
                 "peak": peak, "peak_kind": f"of {peak_kind}", "unit": "GB/s",
                 "frac": kernels[dom]["frac"], "traffic": traffic, "traffic_note": traffic_note,
-                "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": kernels[dom]["frac_of_nominal"],
+                "nominal_peak": NOMINAL_HBM_GBS,
                 "step_frac": m.step_bytes / (ms_step * 1e-3) / 1e9 / peak,
                 "step_frac_of_nominal": m.step_bytes / (ms_step * 1e-3) / 1e9 / NOMINAL_HBM_GBS,
                 # the target is stated against the nominal rate: which kernels of this run meet it
@@ -580,9 +611,14 @@ def run_b200(args):
             "config": cfg,
             "clocks": clock_info, "e2e": e2e, "gpu_launches": int(gpu_launches),
             "roofline": roofline, "kernels": kernels, "cpu_baseline": cpu_baseline,
-            "device_status": int(status), "configs": configs,
+            "device_status": int(status),
         }
-        print(json.dumps(line), flush=True)
+        if configs is not None:
+            line["configs"] = [config_brief(rec) for rec in configs]
+            if args.records:
+                with open(args.records, "w") as f:
+                    f.writelines(json.dumps(rec) + "\n" for rec in configs)
+        print(printed_line(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
 

@@ -50,3 +50,17 @@ def test_two_full_passes_keep_a_record_each(monkeypatch):
     q = _Handle(1 << 20, 2, 0, 4 << 20)
     t = bench.kernel_table(_profile(absmax=0.8, quantize=0.2), w, "worker", q, 0.0, 6500.0)
     assert set(t) == {"absmax", "quantize"} and all(k["achieved_gbs"] > 0 for k in t.values())
+
+
+def test_the_printed_line_is_short_enough_to_be_read_back():
+    rec = {"workload": "resnet18_qg_qx_k1", "n_workers": 8, "placement": "worker", "weight_decay": 5e-4,
+           "weight_feedback": True, "ms_per_step": 0.0123456789, "step_frac": 0.123456}
+    line = {"metric": bench.METRIC, "value": 391295412345.678, "config": {"text": "x" * 800},
+            "kernels": {k: {"ms_per_launch": 1.23456789, "frac": 0.123456789} for k in "abcdef"},
+            "configs": [bench.config_brief(rec)] * 20}
+    short = bench.printed_line(line)
+    assert len(short) < bench.LINE_CHARS and len(bench.json.loads(short)["configs"]) == 20
+    short = bench.printed_line({**line, "configs": line["configs"] * 5})
+    back = bench.json.loads(short)
+    assert len(short) < bench.LINE_CHARS and 20 < len(back["configs"]) < 100
+    assert back["metric"] == bench.METRIC and abs(back["value"] / line["value"] - 1) < 1e-5
