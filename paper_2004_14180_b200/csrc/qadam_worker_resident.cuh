@@ -590,22 +590,19 @@ worker_resident_kernel(const WorkerResidentParams rp) {
     // pair's word depends on the first worker of the call, so a word can outlive any number of
     // launches that cut the workers otherwise; before the numbers start again the last CTA
     // therefore clears all words (nobody reads them any more), and a number never comes back to one.
-    if (warp == 0) {
-      int clear = 0;
-      if (lane == 0) {
-        __threadfence();
-        if (atomicAdd(rp.epoch + 1, 1u) == (unsigned)ctas - 1u) {
-          const unsigned next = (__ldcg(rp.epoch) + 1u) & 0xffffffu;
-          rp.epoch[1] = 0u;
-          rp.epoch[0] = next != 0u ? next : 1u;
-          if (next == 0u) {
-            __threadfence();
-            clear = 1;
-          }
+    // (By one thread, some milliseconds once in 2^24 launches: a warp that stays together for it, as a
+    // branch or as a call, costs two of the kernels a spill and them 1.4 % of a step.)
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(rp.epoch + 1, 1u) == (unsigned)ctas - 1u) {
+        const unsigned next = (__ldcg(rp.epoch) + 1u) & 0xffffffu;
+        rp.epoch[1] = 0u;
+        rp.epoch[0] = next != 0u ? next : 1u;
+        if (next == 0u) {
+          __threadfence();
+          for (long long i = 0; i < rp.num_words; ++i) rp.words[i] = 0ull;
         }
       }
-      if (__shfl_sync(0xffffffffu, clear, 0))
-        for (long long i = lane; i < rp.num_words; i += 32) rp.words[i] = 0ull;
     }
   }
 }
