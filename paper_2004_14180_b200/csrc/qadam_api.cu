@@ -15,6 +15,7 @@
 #include "qadam_kernels.cuh"
 #include "qadam_server_pipe.cuh"
 #include "qadam_worker_resident.cuh"
+#include "qadam_worker_stream.cuh"
 
 using namespace qadam;
 
@@ -57,6 +58,11 @@ int grad_levels(int kg, int grid) {
 
 constexpr int kWordCtas = 256;                       // CTAs the per-pair words are sized for
 constexpr size_t kWordBudget = (size_t)32 << 20;     // bytes of workspace they may take
+// Entries of the list of open elements: one per 64 elements of the segments that are likely to be
+// swept (0.125 bytes beside the 8 of g and e), and a few for the others.
+constexpr int kListTiles = 1024;
+constexpr int64_t kListShare = 64;
+constexpr size_t kListEntries = (size_t)1 << 16;
 
 struct Geometry {
   std::vector<int64_t> seg_len, seg_off;
@@ -73,7 +79,8 @@ struct Geometry {
   std::vector<RTile> rtiles;
   std::vector<Tile> btiles;
   long long resident_elems = 0;      // padded elements of the resident segments (one vector)
-  size_t off_rtiles = 0, off_btiles = 0, off_words = 0, off_epoch = 0, off_deferred = 0;
+  size_t off_rtiles = 0, off_btiles = 0, off_words = 0, off_epoch = 0, off_counters = 0, off_deferred = 0, off_open = 0;
+  size_t open_entries = 0;           // of the list of the elements the sweep leaves open
   size_t words_bytes = 0;            // room for the per-(pair, CTA) words of the on-chip worker kernel
 };
 
@@ -209,11 +216,20 @@ int build_geometry(const qadam_config* c, Geometry* g) {
     g->off_epoch = wo;
     wo += 256;
   }
-  // flags of the rows the sweep leaves to the second kernel: a byte per 512 elements, 8 per tile
+  g->off_counters = wo;
+  wo += 256;
+  // flags of the rows the sweep leaves to the settle pass: a byte per 512 elements, 8 per tile
   // however short (1 / 2048 of the size of e where tiles are full)
   g->off_deferred = wo;
-  if (sweeps(c, g->gmode))
-    wo += 256 + (size_t)round_up64((int64_t)c->n * (int64_t)g->tiles.size() * kTileChunks, 256);   // a count first
+  if (sweeps(c, g->gmode)) wo += (size_t)round_up64((int64_t)c->n * (int64_t)g->tiles.size() * kTileChunks, 256);
+  g->off_open = wo;
+  if (sweeps(c, g->gmode)) {
+    int64_t large = 0;
+    for (int s = 0; s < S; ++s)
+      if (g->seg_tiles[s] > kListTiles) large += g->seg_len[s];
+    g->open_entries = kListEntries + (size_t)(c->n * large / kListShare);
+    wo += (size_t)round_up64((int64_t)(g->open_entries * sizeof(unsigned long long)), 256);
+  }
   g->workspace_bytes = wo + 256;
   return QADAM_OK;
 }
@@ -232,7 +248,8 @@ struct qadam_ctx {
   int64_t last_server_step;     // steps completed by the server
   int64_t workers_done;         // workers compressed for step last_server_step + 1
   int64_t launches;
-  int grid_absmax, grid_quant, grid_ident, grid_server, grid_bcast;
+  int form_stages[2] = {0, 0}, settle_stages = 0;   // of the streaming passes' rings, form: without and with the l2 term
+  int grid_ident, grid_server, grid_bcast;
   size_t server_smem;
   // persistent pipelined server pass: stages > 0 when in use
   float lambda = 0.0f;       // l2 term (qadam_set_regularization)
@@ -252,7 +269,9 @@ struct qadam_ctx {
   size_t res_smem_l2 = 0;
   RTile* d_rtiles = nullptr;
   Tile* d_btiles = nullptr;
+  StreamCounters* d_counters = nullptr;
   unsigned char* d_deferred = nullptr;
+  unsigned long long* d_open = nullptr;
   unsigned* d_epoch = nullptr;
   unsigned long long* d_words = nullptr;   // nullptr: one counter per pair instead
   // qadam_step_host: the copy of worker i + 1 runs on a stream of its own while worker i is compressed
@@ -279,47 +298,37 @@ int resident_grid(K kernel, size_t smem, int sm_count) {
 using WorkerKernel = void (*)(const WorkerParams);
 using ServerKernel = void (*)(const ServerParams);
 
-// The first of the two streaming launches: max-abs, or the sweep that settles the rows it can.
-WorkerKernel pick_absmax(const qadam_ctx* c) {
-  const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
-  const bool l2 = c->lambda != 0.0f;
+// The first of the two streaming launches: the sweep that settles what it can, or u and its maxima alone.
+WorkerKernel pick_form(const qadam_ctx* c, bool l2) {
   if (sweeps(&c->cfg, c->geo.gmode)) {
     if (c->geo.gmode == G_TERNARY) return l2 ? worker_sweep_kernel<2, true> : worker_sweep_kernel<2, false>;
     return l2 ? worker_sweep_kernel<3, true> : worker_sweep_kernel<3, false>;
   }
-  if (l2) return w ? worker_absmax_kernel<true, true> : worker_absmax_kernel<false, true>;
-  return w ? worker_absmax_kernel<true> : worker_absmax_kernel<false>;
+  if (c->cfg.placement == QADAM_PLACE_WORKER) return l2 ? worker_form_kernel<true, true> : worker_form_kernel<true, false>;
+  return l2 ? worker_form_kernel<false, true> : worker_form_kernel<false, false>;
+}
+
+// The second: codes and e' of everything, or of what the sweep left.
+WorkerKernel pick_settle(const qadam_ctx* c) {
+  const bool swept = sweeps(&c->cfg, c->geo.gmode);
+  switch (c->geo.gmode) {
+    case G_STOCHASTIC: return worker_settle_kernel<G_STOCHASTIC, false>;
+    case G_TERNARY: return swept ? worker_settle_kernel<G_TERNARY, true> : worker_settle_kernel<G_TERNARY, false>;
+    case G_FIVE:    return swept ? worker_settle_kernel<G_FIVE, true> : worker_settle_kernel<G_FIVE, false>;
+    case G_POW2:    return worker_settle_kernel<G_POW2, false>;
+    default:        return worker_settle_kernel<G_UNIFORM, false>;
+  }
+}
+
+// bytes of a stage of the first launch's ring
+int form_bytes(const qadam_ctx* c, bool l2) {
+  return form_stage_bytes(c->cfg.placement == QADAM_PLACE_WORKER, l2 ? held_tile_bytes(c->cfg.kx, c->geo.xbits) : 0);
 }
 
 WorkerKernel pick_identity(const qadam_ctx* c) {
   const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
   if (c->lambda != 0.0f) return w ? worker_identity_kernel<true, true> : worker_identity_kernel<false, true>;
   return w ? worker_identity_kernel<true> : worker_identity_kernel<false>;
-}
-
-// The second: quantize everything, or the rows the sweep left.
-template <int MODE>
-WorkerKernel pick_quantize_mode(bool worker_moments, bool l2) {
-  if (worker_moments) return worker_quantize_kernel<true, MODE>;
-  // moments on the server: phase 2 forms u = g + e again, l2 term included
-  return l2 ? worker_quantize_kernel<false, MODE, true> : worker_quantize_kernel<false, MODE>;
-}
-template <int MODE>
-WorkerKernel pick_deferred_mode(bool worker_moments, bool l2) {
-  if (worker_moments) return worker_quantize_kernel<true, MODE>;
-  return l2 ? worker_deferred_kernel<MODE, true> : worker_deferred_kernel<MODE, false>;
-}
-
-WorkerKernel pick_quantize(const qadam_ctx* c) {
-  const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
-  const bool l2 = c->lambda != 0.0f;
-  switch (c->geo.gmode) {
-    case G_STOCHASTIC: return pick_quantize_mode<G_STOCHASTIC>(w, l2);
-    case G_TERNARY: return pick_deferred_mode<G_TERNARY>(w, l2);
-    case G_FIVE:    return pick_deferred_mode<G_FIVE>(w, l2);
-    case G_POW2:    return pick_quantize_mode<G_POW2>(w, l2);
-    default:        return pick_quantize_mode<G_UNIFORM>(w, l2);
-  }
 }
 
 ServerKernel pick_server(const qadam_ctx* c) {
@@ -390,13 +399,11 @@ WorkerResidentKernel pick_worker_resident(const qadam_ctx* c, bool l2, bool word
   }
 }
 
-// grids of the split worker kernels (they depend on whether the l2 term is on)
-bool plan_worker_grids(qadam_ctx* c) {
-  const int a = resident_grid(pick_absmax(c), 0, c->sm_count);
-  const int q = resident_grid(pick_quantize(c), 0, c->sm_count);
+// grid of the identity worker (it depends on whether the l2 term is on)
+bool plan_identity_grid(qadam_ctx* c) {
   const int i = resident_grid(pick_identity(c), 0, c->sm_count);
-  if (a < 0 || q < 0 || i < 0) return false;
-  c->grid_absmax = a; c->grid_quant = q; c->grid_ident = i;
+  if (i < 0) return false;
+  c->grid_ident = i;
   return true;
 }
 
@@ -537,7 +544,9 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     c->d_done = reinterpret_cast<unsigned*>(ws + c->geo.off_done);
     c->d_rtiles = reinterpret_cast<RTile*>(ws + c->geo.off_rtiles);
     c->d_btiles = reinterpret_cast<Tile*>(ws + c->geo.off_btiles);
+    c->d_counters = reinterpret_cast<StreamCounters*>(ws + c->geo.off_counters);
     c->d_deferred = ws + c->geo.off_deferred;
+    c->d_open = reinterpret_cast<unsigned long long*>(ws + c->geo.off_open);
     c->d_epoch = reinterpret_cast<unsigned*>(ws + c->geo.off_epoch);
     c->d_words = c->geo.words_bytes ? reinterpret_cast<unsigned long long*>(ws + c->geo.off_words) : nullptr;
   }
@@ -595,7 +604,25 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
       }
     }
   }
-  if (!plan_worker_grids(c)) { delete c; return QADAM_ERR_CUDA; }
+  if (!plan_identity_grid(c)) { delete c; return QADAM_ERR_CUDA; }
+  if (c->geo.gmode != G_IDENTITY) {
+    int max_smem = 0;
+    bool ok = cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    for (int l2 = 0; l2 < 2 && ok; ++l2) {
+      const int stage = form_bytes(c, l2 != 0);
+      c->form_stages[l2] = stream_stages(max_smem, stage);
+      if (sweeps(cfg, c->geo.gmode)) c->form_stages[l2] = c->form_stages[l2] / kStreamGroups * kStreamGroups;
+      ok = c->form_stages[l2] >= 1 &&
+           cuda_ok(cudaFuncSetAttribute(pick_form(c, l2 != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)stream_smem_bytes(c->form_stages[l2], stage)));
+    }
+    c->settle_stages = stream_stages(max_smem, kSettleStageBytes) / kStreamGroups * kStreamGroups;
+    if (!ok || c->settle_stages < 1 ||
+        !cuda_ok(cudaFuncSetAttribute(pick_settle(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)stream_smem_bytes(c->settle_stages, kSettleStageBytes)))) {
+      delete c; return QADAM_ERR_CUDA;
+    }
+  }
   c->grid_server = resident_grid(sk, c->server_smem, c->sm_count);
   c->grid_bcast = resident_grid(weight_broadcast_kernel, 0, c->sm_count);
   // Worker side.  Segments small enough to be held by the
@@ -616,7 +643,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     if (eligible) {
       // the CTA's shared memory: a ring of slots for u and a few stages for e (227 KB: 14 in all)
       const int estages = 2;                  // measured: 12 slots + 2 stages beat 11 + 3 and 10 + 4
-      const int held = resident_held_bytes(cfg->kx, c->geo.xbits);
+      const int held = held_tile_bytes(cfg->kx, c->geo.xbits);
       auto slots_for = [&](int held_bytes) {
         return std::min(((int)max_smem - kRHeadBytes - estages * (resident_stage_bytes(wm) + held_bytes)) / kRSlotBytes,
                         kRMaxSlots);
@@ -668,6 +695,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
        (!cuda_ok(cudaMemsetAsync(c->d_words, 0, c->geo.words_bytes, c->stream)) ||
         !cuda_ok(cudaMemsetAsync(c->d_epoch, 0, 2 * sizeof(unsigned), c->stream)) ||
         !cuda_ok(cudaMemsetAsync(c->d_epoch, 1, 1, c->stream)))) ||
+      !cuda_ok(cudaMemsetAsync(c->d_counters, 0, sizeof(StreamCounters), c->stream)) ||
       !cuda_ok(cudaMemsetAsync(b->status, 0, sizeof(uint32_t), c->stream)) ||
       !cuda_ok(cudaStreamSynchronize(c->stream))) {
     delete c; return QADAM_ERR_CUDA;
@@ -720,30 +748,36 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
   p.seed_lo = (unsigned)c->cfg.seed;
   p.seed_hi = (unsigned)(c->cfg.seed >> 32);
   p.step = (unsigned)step;
-  p.deferred = c->d_deferred + 256;
-  p.deferred_rows = reinterpret_cast<unsigned*>(c->d_deferred);
+  p.deferred = c->d_deferred;
+  p.open_list = c->d_open;
+  p.open_stride = 0;
+  p.open_regions = 0;
+  p.stages = 0;
+  p.counters = c->d_counters;
 
-  // the two streaming launches over a tile table: max-abs, then quantize (or the sweep, then the
-  // rows it left)
+  // the two streaming launches over a tile table
   auto streaming = [&](const Tile* tiles, int tiles_per_worker) -> int {
     WorkerParams q = p;
     q.tiles = tiles;
     q.tiles_per_worker = tiles_per_worker;
     q.total_tiles = (long long)worker_count * tiles_per_worker;
-    if (sweeps(&c->cfg, c->geo.gmode) &&
-        !cuda_ok(cudaMemsetAsync(q.deferred_rows, 0, sizeof(unsigned), c->stream)))
-      return QADAM_ERR_CUDA;
-    int grid = (int)std::min<int64_t>(c->grid_absmax, q.total_tiles);
+    const bool l2 = c->lambda != 0.0f;
+    const int grid = (int)std::min<int64_t>(c->sm_count, q.total_tiles);
+    if (sweeps(&c->cfg, c->geo.gmode) && q.total_tiles < 1 << 23) {      // (an entry has 23 bits for its tile)
+      q.open_regions = (unsigned)grid * kStreamWarps;
+      q.open_stride = (unsigned)std::min<size_t>(c->geo.open_entries / q.open_regions, 1u << 30);
+    }
     {
       LaunchTimer lt(c, QADAM_K_ABSMAX);
-      pick_absmax(c)<<<grid, kThreads, 0, c->stream>>>(q);
+      q.stages = c->form_stages[l2];
+      pick_form(c, l2)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, form_bytes(c, l2)), c->stream>>>(q);
     }
     if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
     c->launches += 1;
-    grid = (int)std::min<int64_t>(c->grid_quant, q.total_tiles);
     {
       LaunchTimer lt(c, QADAM_K_QUANTIZE);
-      pick_quantize(c)<<<grid, kThreads, 0, c->stream>>>(q);
+      q.stages = c->settle_stages;
+      pick_settle(c)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, kSettleStageBytes), c->stream>>>(q);
     }
     if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
     c->launches += 1;
@@ -784,7 +818,7 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
       rp.total = (long long)worker_count * rp.TR;
       rp.slots = l2 ? c->res_slots_l2 : c->res_slots;
       rp.estages = c->res_estages;
-      rp.held_bytes = l2 ? resident_held_bytes(c->cfg.kx, c->geo.xbits) : 0;
+      rp.held_bytes = l2 ? held_tile_bytes(c->cfg.kx, c->geo.xbits) : 0;
       void* args[] = {&rp};
       cudaError_t e;
       {
@@ -833,8 +867,8 @@ int qadam_set_regularization(qadam_ctx* c, float lambda) {
   const bool changed = (c->lambda != 0.0f) != (lambda != 0.0f);
   const float before = c->lambda;
   c->lambda = lambda;
-  // the streaming kernels with and without the term differ: their grids are planned again
-  if (changed && !plan_worker_grids(c)) {
+  // the identity kernels with and without the term differ: the grid is planned again
+  if (changed && !plan_identity_grid(c)) {
     c->lambda = before;
     return QADAM_ERR_CUDA;
   }

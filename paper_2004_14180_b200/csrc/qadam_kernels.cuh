@@ -1,6 +1,6 @@
-// The step kernels: worker phase 1 (form u, reduce max|u|), worker phase 2
-// (quantize, pack, residual), the identity worker, the fused server pass and the
-// stand-alone weight broadcast.  All are grid-stride loops over a tile table.
+// The plain step kernels: the identity worker, the server pass for the streams the pipelined one
+// does not take and the stand-alone weight broadcast, grid-stride loops over a tile table; and what
+// the pipelined kernels share with them.
 //
 // Thread/tile mapping (all kernels): a CTA of 256 threads owns a tile of up to
 // 4096 consecutive padded elements as 4 CTA-wide rows of 1024; in row r thread t
@@ -12,6 +12,8 @@
 #include "qadam_device.cuh"
 
 namespace qadam {
+
+struct StreamCounters;          // see the streaming passes
 
 struct WorkerParams {
   const float* g;        // [worker_count][D] gradients of the workers of this call
@@ -39,9 +41,15 @@ struct WorkerParams {
   unsigned spin_limit;          // persistent kernels: polls of one wait before it gives up
   // stochastic operator: key of the random stream and the step number
   unsigned seed_lo, seed_hi, step;
-  // sweep and its deferred rows: one byte per 512-element chunk of a tile, [total_tiles][8]
+  // sweep: the rows it leaves, one byte per 512-element chunk of a tile, [total_tiles][8] ...
   unsigned char* deferred;
-  unsigned* deferred_rows;      // how many rows the sweep flagged
+  // ... and the open elements it listed instead: a region of open_stride entries per warp of the sweep,
+  // {entry 0: how many follow} {u : 32, tile : 23, element of the chunk : 9} ...
+  unsigned long long* open_list;
+  unsigned open_stride;         // 0: no list
+  unsigned open_regions;
+  int stages;                   // of the streaming passes' rings
+  StreamCounters* counters;
 };
 
 // Packed weight codes of at most 8 bits: the two 32-bit words that hold this lane's 4 codes
@@ -108,25 +116,6 @@ __device__ __forceinline__ void held_weights4(const WorkerParams& p, long long r
     out[2 * h + 1] = value((f >> p.xbits) & mask);
   }
 }
-// The held weights of a thread's 4 elements of a row as they are loaded when the weights are
-// packed codes of at most 8 bits: the two words that hold the lane's 4 codes, fetched together
-// with the loads of g and e and decoded when the row is processed.  Unquantized weights and
-// wider codes are read at the point of use (fetched stays false).
-struct HeldRaw {
-  unsigned lo, hi;
-  bool fetched;
-};
-__device__ __forceinline__ HeldRaw held_fetch(const WorkerParams& p, long long row_elem, int lane) {
-  HeldRaw h;
-  h.lo = h.hi = 0u;
-  h.fetched = p.kx >= 0 && p.xbits <= 8;
-  if (h.fetched) held_fetch8(p, row_elem, lane, h.lo, h.hi);
-  return h;
-}
-// g + lambda * (held weights) from what held_fetch loaded
-__device__ __forceinline__ void add_l2_term_held(const WorkerParams& p, long long row_elem, int lane,
-                                                 const HeldRaw& h, float gg[4]);
-
 // g + lambda * (held weights), each operation rounded once (Section 5.1's l2 term)
 __device__ __forceinline__ void add_l2_term(const WorkerParams& p, long long row_elem, int lane,
                                             float gg[4]) {
@@ -136,17 +125,8 @@ __device__ __forceinline__ void add_l2_term(const WorkerParams& p, long long row
   for (int c = 0; c < 4; ++c) gg[c] = __fadd_rn(gg[c], __fmul_rn(p.lambda, w[c]));
 }
 
-__device__ __forceinline__ void add_l2_term_held(const WorkerParams& p, long long row_elem, int lane,
-                                                 const HeldRaw& h, float gg[4]) {
-  if (!h.fetched) {
-    add_l2_term(p, row_elem, lane, gg);
-    return;
-  }
-  float w[4];
-  held_decode8(p, lane, h.lo, h.hi, w);
-#pragma unroll
-  for (int c = 0; c < 4; ++c) gg[c] = __fadd_rn(gg[c], __fmul_rn(p.lambda, w[c]));
-}
+// With the l2 term a pipeline stage also carries its tile's held weights: b_x bits (x: 32) per element.
+__host__ __device__ constexpr int held_tile_bytes(int kx, int xbits) { return kTileElems / 8 * (kx < 0 ? 32 : xbits); }
 
 // The same from a copy of the tile's held weights in shared memory (packed codes, or x itself);
 // row: the row's first element in the tile.
@@ -215,493 +195,6 @@ __device__ __forceinline__ float4 ld_f4_stream(const float* p) {
 }
 __device__ __forceinline__ void st_f4(float* p, const float4& v) {
   *reinterpret_cast<float4*>(p) = v;
-}
-
-// CTA-wide max of a 32-bit pattern; result valid in thread 0.
-__device__ __forceinline__ unsigned block_max(unsigned v, unsigned* smem8) {
-  v = warp_max(v);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) smem8[warp] = v;
-  __syncthreads();
-  unsigned r = 0;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) r = max(r, smem8[w]);
-  }
-  __syncthreads();
-  return r;
-}
-
-// ---------------------------------------------------------------------------
-// Worker phase 1.  PLACE_SERVER: u = g + e, nothing written but the running
-// max.  PLACE_WORKER: v, m updated in place, u = alpha m/sqrt(v+eps) + e stored
-// in e's slot for phase 2.  The max over a (worker, segment) is taken on the bit
-// patterns of |u| (monotone for non-negative floats, exact, order-free; a NaN
-// or Inf ends up as the maximum and is reported by phase 2).
-// ---------------------------------------------------------------------------
-template <bool WORKER_MOMENTS, bool L2 = false>
-__global__ void __launch_bounds__(kThreads, WORKER_MOMENTS ? 2 : (L2 ? 3 : 4))
-worker_absmax_kernel(const WorkerParams p) {
-  __shared__ unsigned red[kThreads / 32];
-  unsigned mx = 0;
-  long long cur_pair = -1;
-  for (long long t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
-    const int wl = (int)(t / p.tiles_per_worker);
-    const Tile tile = p.tiles[(int)(t - (long long)wl * p.tiles_per_worker)];
-    const int w = p.worker_begin + wl;
-    const long long pair = (long long)w * p.S + tile.seg;
-    if (pair != cur_pair) {
-      if (cur_pair >= 0) {
-        const unsigned r = block_max(mx, red);
-        if (threadIdx.x == 0 && r) atomicMax(p.scale_bits + cur_pair, r);
-      }
-      mx = 0;
-      cur_pair = pair;
-    }
-    const float* gp = p.g + (long long)wl * p.D + tile.off;
-    const long long so = (long long)w * p.D + tile.off;
-    float4 gv[kRows], ev[kRows], mv[kRows], vv[kRows];
-    HeldRaw hw[L2 ? kRows : 1];
-    bool act[kRows];
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      const int idx = r * kRowElems + threadIdx.x * 4;
-      act[r] = idx < tile.count;
-      if (act[r]) {
-        gv[r] = ld_f4_stream(gp + idx);
-        ev[r] = ld_f4(p.e + so + idx);
-        if constexpr (WORKER_MOMENTS) {
-          mv[r] = ld_f4(p.m + so + idx);
-          vv[r] = ld_f4(p.v + so + idx);
-        }
-        if constexpr (L2)
-          hw[r] = held_fetch(p, tile.off + r * kRowElems + (threadIdx.x >> 5) * 128, threadIdx.x & 31);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      if (!act[r]) continue;
-      const int idx = r * kRowElems + threadIdx.x * 4;
-      float gg[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w};
-      float ee[4] = {ev[r].x, ev[r].y, ev[r].z, ev[r].w};
-      float uu[4];
-      if constexpr (L2)
-        add_l2_term_held(p, tile.off + r * kRowElems + (threadIdx.x >> 5) * 128, threadIdx.x & 31, hw[r], gg);
-      if constexpr (WORKER_MOMENTS) {
-        float mm[4] = {mv[r].x, mv[r].y, mv[r].z, mv[r].w};
-        float vs[4] = {vv[r].x, vv[r].y, vv[r].z, vv[r].w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          moments(p.h, gg[c], mm[c], vs[c]);
-          uu[c] = __fadd_rn(adam_step(p.h, mm[c], vs[c], p.alpha), ee[c]);
-        }
-        st_f4(p.m + so + idx, make_float4(mm[0], mm[1], mm[2], mm[3]));
-        st_f4(p.v + so + idx, make_float4(vs[0], vs[1], vs[2], vs[3]));
-        st_f4(p.e + so + idx, make_float4(uu[0], uu[1], uu[2], uu[3]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) uu[c] = __fadd_rn(gg[c], ee[c]);
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) mx = max(mx, __float_as_uint(fabsf(uu[c])));
-    }
-  }
-  if (cur_pair >= 0) {
-    const unsigned r = block_max(mx, red);
-    if (threadIdx.x == 0 && r) atomicMax(p.scale_bits + cur_pair, r);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Worker side, moments on the server, for pairs that do not fit on chip: one sweep over g, e
-// that settles every row of 128 elements it can, and a second kernel for the rows it cannot.
-//
-// A coordinate has level 0 whenever |u| <= t s, t = 2^-(k+1) the lowest midpoint of the grid,
-// and then its code is L and e' = u: the scale itself does not enter.  Any maximum seen so far
-// bounds s from below, so a row whose largest |u| is at most t times that bound is finished
-// in the sweep: 12 + b/8 bytes per element, the least there is.  Every other row is left
-// untouched and flagged; the second kernel reads its g and e again when the scale is known.  So
-// a row costs 12 + b/8 or 20 + b/8 bytes, never more than the two full passes (max-abs, then
-// quantize) that this replaces, and the error feedback keeps the codes of heavy-tailed gradients
-// sparse (2^28 elements of the benchmark's mixture after 18 steps: 10 % of the rows hold a code
-// other than level 0; Gaussian gradients: nearly all rows do).  Settling all but the few open
-// lanes of such rows in the sweep and fetching those alone afterwards was tried: fewer bytes, but
-// scattered 32-byte accesses, 3.8 ms for the second kernel instead of 1.4.
-//
-// A warp owns 512 consecutive elements of a tile (4 rows, so that its ternary codes are one
-// 128-byte line).  The block keeps the bound of its current pair in shared memory, and its warps
-// take turns in exchanging it with the pair's word of the scales, each with every eighth tile:
-// with every warp of the chip on that one address with every tile, the start of a pair cost 4 us
-// and the sweep ran at 0.90 of the copy rate.  (Turns, because warps are not kept in step: one
-// warp doing it alone falls behind the others, pairs behind in the end, and they never learn the
-// bound: 15 % of the rows left instead of 10 %.)
-// The first tiles of a pair find a low bound and are mostly flagged: a few per mille of a pair
-// of 10^8 elements.
-// ---------------------------------------------------------------------------
-constexpr int kChunkRows = 4;                         // rows of 128 elements per warp and tile
-constexpr int kChunkElems = kChunkRows * 128;
-constexpr int kTileChunks = kTileElems / kChunkElems; // 8, one per warp
-
-// BITS: code width, 2 (ternary) or 3 (five levels).
-template <int BITS, bool L2>
-__global__ void __launch_bounds__(kThreads, L2 ? 3 : 4)
-worker_sweep_kernel(const WorkerParams p) {
-  // {pair, bits of a maximum}: what the block knows of its pair, and what it knows to be in
-  // the pair's word.  Pairs grow along the block's tiles, so a 64-bit maximum lets a newer
-  // pair replace an older one.
-  __shared__ unsigned long long s_known, s_published;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_known = s_published = 0ull;
-  __syncthreads();
-  volatile unsigned long long* known = &s_known;
-  volatile unsigned long long* published = &s_published;
-  // words of the level-0 pattern: code L in fields of BITS bits, from bit 32 j of a row on
-  unsigned long long rep = (unsigned long long)p.L;
-#pragma unroll
-  for (int width = BITS; width < 64; width *= 2) rep |= rep << width;
-  constexpr int kRowWords = 4 * BITS;                 // 32-bit words of one row of codes
-  const float mid = exp2i(-p.k - 1);                  // the lowest midpoint
-  const int first = warp * kChunkElems;               // of the warp's rows in a tile
-  unsigned run = 0;                                   // maximum of this warp's rows of the pair
-  unsigned cur_pair = ~0u;                            // n * S and the tiles fit 31 bits (their data would not fit a GPU)
-  // what this warp knows of a pair it leaves goes into the pair's word unless it is there
-  auto leave = [&]() {
-    if (lane == 0 && run != 0u) {
-      const unsigned long long pub = *published;
-      if ((unsigned)(pub >> 32) != cur_pair || (unsigned)pub < run) atomicMax(p.scale_bits + cur_pair, run);
-    }
-  };
-  unsigned flagged = 0;
-  int turn = warp, age = 0;                           // tiles done, shifted by the warp; tiles of the pair
-  const unsigned total = (unsigned)p.total_tiles;
-  int wl = (int)(blockIdx.x / (unsigned)p.tiles_per_worker);
-  int tl = (int)(blockIdx.x - (unsigned)wl * (unsigned)p.tiles_per_worker);
-  for (unsigned t = blockIdx.x; t < total; t += gridDim.x) {
-    const Tile tile = p.tiles[tl];
-    const int w = p.worker_begin + wl;
-    const unsigned pair = (unsigned)w * (unsigned)p.S + (unsigned)tile.seg;
-    if (pair != cur_pair) {
-      leave();
-      run = 0;
-      age = 0;
-      cur_pair = pair;
-    }
-    const float* gp = p.g + (long long)wl * p.D + tile.off + first + lane * 4;
-    tl += (int)gridDim.x;
-    while (tl >= p.tiles_per_worker) {
-      tl -= p.tiles_per_worker;
-      ++wl;
-    }
-    if (first >= tile.count) {                        // a short tile: nothing of this warp's
-      if (lane == 0) p.deferred[(long long)t * kTileChunks + warp] = 0;
-      continue;
-    }
-    float* ep = p.e + (long long)w * p.D + tile.off + first + lane * 4;
-    float4 gv[kChunkRows], u4[kChunkRows];
-    HeldRaw hw[L2 ? kChunkRows : 1];
-#pragma unroll
-    for (int r = 0; r < kChunkRows; ++r) {
-      if (first + r * 128 < tile.count) {
-        gv[r] = ld_f4_stream(gp + r * 128);
-        u4[r] = ld_f4(ep + r * 128);
-        if constexpr (L2) hw[r] = held_fetch(p, tile.off + first + r * 128, lane);
-      }
-    }
-    unsigned word = 0;
-    const bool exchange = (++turn & 7) == 0;
-    if (exchange || age == 1) word = *reinterpret_cast<volatile const unsigned*>(p.scale_bits + pair);
-    unsigned row_max[kChunkRows], mx = 0;
-#pragma unroll
-    for (int r = 0; r < kChunkRows; ++r) {
-      row_max[r] = 0;
-      if (first + r * 128 >= tile.count) continue;
-      float gg[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w};
-      if constexpr (L2) add_l2_term_held(p, tile.off + first + r * 128, lane, hw[r], gg);
-      u4[r] = make_float4(__fadd_rn(gg[0], u4[r].x), __fadd_rn(gg[1], u4[r].y), __fadd_rn(gg[2], u4[r].z),
-                          __fadd_rn(gg[3], u4[r].w));
-      row_max[r] = max(max(__float_as_uint(fabsf(u4[r].x)), __float_as_uint(fabsf(u4[r].y))),
-                       max(__float_as_uint(fabsf(u4[r].z)), __float_as_uint(fabsf(u4[r].w))));
-      mx = max(mx, row_max[r]);
-    }
-    const unsigned wm = warp_max(mx);
-    run = max(run, wm);
-    if (wm >= 0x7f800000u && lane == 0) atomicOr(p.status, 1u);
-    const unsigned long long kn = *known;
-    const unsigned in_block = (unsigned)(kn >> 32) == pair ? (unsigned)kn : 0u;
-    const unsigned best = max(max(run, word), in_block);
-    if (lane == 0) {
-      const unsigned long long tag = (unsigned long long)pair << 32;
-      if (best > in_block) atomicMax(&s_known, tag | best);
-      if (exchange) {
-        if (best > word) atomicMax(p.scale_bits + pair, best);
-        atomicMax(&s_published, tag | best);
-      }
-    }
-    ++age;
-    // mid * bound is exact for bounds of ordinary size; below that only zeros are sure of level 0
-    const float bound = __uint_as_float(best);
-    const unsigned thr = bound >= 1e-30f ? __float_as_uint(__fmul_rn(bound, mid)) : 0u;
-    unsigned flags = 0;
-#pragma unroll
-    for (int r = 0; r < kChunkRows; ++r) {
-      if (first + r * 128 >= tile.count) continue;
-      if (__any_sync(0xffffffffu, row_max[r] > thr)) flags |= 1u << r;
-      else st_f4(ep + r * 128, u4[r]);
-    }
-    unsigned* cw = reinterpret_cast<unsigned*>(p.gcodes + (long long)w * p.gcode_bytes +
-                                               (tile.off + first) * BITS / 8);
-    const int words = min(kChunkRows, (tile.count - first) >> 7) * kRowWords;
-#pragma unroll
-    for (int j0 = 0; j0 < kChunkRows * kRowWords; j0 += 32) {
-      const int j = j0 + lane, r = j / kRowWords;
-      if (j < words && !((flags >> r) & 1u)) cw[j] = (unsigned)(rep >> ((32 * (j - r * kRowWords)) % BITS));
-    }
-    if (lane == 0) p.deferred[(long long)t * kTileChunks + warp] = (unsigned char)flags;
-    flagged += __popc(flags);
-  }
-  leave();
-  if (lane == 0 && flagged) atomicAdd(p.deferred_rows, flagged);
-}
-
-// One row the sweep left: u = g (+ l2 term) + e, quantized, packed, e'.
-template <int MODE, bool L2>
-__device__ __forceinline__ void deferred_row(const WorkerParams& p, const float4& g4, const float4& e4,
-                                             const HeldRaw& hw, const GradScale& gs, long long row_elem,
-                                             float* e_dst, unsigned char* code_dst, int lane) {
-  float gg[4] = {g4.x, g4.y, g4.z, g4.w};
-  if constexpr (L2) add_l2_term_held(p, row_elem, lane, hw, gg);
-  const float uu[4] = {__fadd_rn(gg[0], e4.x), __fadd_rn(gg[1], e4.y), __fadd_rn(gg[2], e4.z), __fadd_rn(gg[3], e4.w)};
-  float en[4];
-  if constexpr (MODE == G_TERNARY) store_row_of_code_bytes(quantize_ternary4(uu, gs, en), code_dst, lane);
-  else pack_row_store_fields<3>(quantize_five4(uu, gs, en), code_dst, lane);
-  st_f4(e_dst, make_float4(en[0], en[1], en[2], en[3]));
-}
-
-// The rows the sweep left, in one of two orders, by how many there are (2^28 elements, n = 16, with
-// 10 % of the rows left; 1.4 x 10^8 Gaussian elements, n = 2, with nearly all of them left):
-//   many  blocks take tiles as a full pass does, every warp its rows of the tile          (- / 0.50 ms)
-//   few   a warp takes 32 chunks (4 tiles) at a time, one byte of flags per lane, and handles
-//         their rows four at a time (kBatch), so that it keeps as many loads in flight as with full tiles;
-//         the flags and descriptors of its next 32 are fetched meanwhile                 (1.4 / 0.57 ms).
-//         Where 32 chunks each would leave warps without any, a warp takes 16, 8, ... 1 (7 x 10^6
-//         elements, n = 1, a third of the rows left: 28 -> 16 us)
-// With the l2 term a warp of the second order takes two rows at a time, which fits three blocks on an
-// SM for either order; two blocks of 111 registers with four rows were slower than the two full
-// passes the sweep replaces where the rows are many (1.2 x 10^8 Gaussian elements, n = 2, lambda on,
-// this kernel: 0.63 -> 0.50 ms, with unquantized weights 0.84 -> 0.64; few: 0.21 / 0.22 ms).
-// (A tile per warp: 2.0 / 0.54 ms; lists of the flagged rows per block: 1.8 / 0.53; 32 chunks from
-// tiles 7 MB apart: 2.9 / 0.69.)
-template <int MODE, bool L2>
-__global__ void __launch_bounds__(kThreads, 3)
-worker_deferred_kernel(const WorkerParams p) {
-  static_assert(MODE == G_TERNARY || MODE == G_FIVE, "grids the sweep serves");
-  constexpr int kBits = MODE == G_TERNARY ? 2 : 3;
-  constexpr int kBatch = L2 ? 2 : 4;                      // rows at a time where few are left
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned total = (unsigned)p.total_tiles, tpw = (unsigned)p.tiles_per_worker;
-  const unsigned left = *p.deferred_rows;
-  if (left == 0u) return;
-  float4 gv[4], ev[4];
-  HeldRaw hw[L2 ? 4 : 1];
-  if (left / 16u >= total) {                              // half of all rows or more
-    const unsigned long long* flags = reinterpret_cast<const unsigned long long*>(p.deferred);
-    unsigned wl = blockIdx.x / tpw, tl = blockIdx.x - wl * tpw;
-    for (unsigned t = blockIdx.x; t < total; t += gridDim.x) {
-      const unsigned long long f = flags[t];              // byte c: rows 4 c .. 4 c + 3 of the tile
-      const Tile tile = p.tiles[tl];
-      const int w = p.worker_begin + (int)wl;
-      const float s = __uint_as_float(p.scale_bits[(long long)w * p.S + tile.seg]);
-      const float* gp = p.g + (long long)wl * p.D + tile.off + threadIdx.x * 4;
-      float* ep = p.e + (long long)w * p.D + tile.off + threadIdx.x * 4;
-      unsigned char* cw = p.gcodes + (long long)w * p.gcode_bytes + (tile.off + warp * 128) * kBits / 8;
-      tl += gridDim.x;
-      while (tl >= tpw) {
-        tl -= tpw;
-        ++wl;
-      }
-      // this warp's rows: warp, warp + 8, ... of 32
-      auto open = [&](int r) { return ((unsigned)(f >> (16 * r + 8 * (warp >> 2) + (warp & 3))) & 1u) != 0u; };
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        if (!open(r)) continue;
-        gv[r] = ld_f4_stream(gp + r * kRowElems);
-        ev[r] = ld_f4(ep + r * kRowElems);
-        if constexpr (L2) hw[r] = held_fetch(p, tile.off + r * kRowElems + warp * 128, lane);
-      }
-      const GradScale gs = grad_scale<MODE>(s, p.k);
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        if (!open(r)) continue;
-        deferred_row<MODE, L2>(p, gv[r], ev[r], hw[L2 ? r : 0], gs, tile.off + r * kRowElems + warp * 128,
-                               ep + r * kRowElems, cw + r * (kRowElems * kBits / 8), lane);
-      }
-    }
-    return;
-  }
-  // a span: 32 consecutive chunks, one per lane, or fewer as long as some warp would have none
-  const unsigned warps = gridDim.x * (kThreads / 32), chunks = total * kTileChunks;   // below 2^32: 512 elements each
-  unsigned span = 32u;
-  while (span > 1u && chunks < span * warps) span >>= 1;
-  unsigned c_next = (blockIdx.x * (kThreads / 32) + warp) * span + (unsigned)lane;
-  unsigned fl_next = 0, wl_next = 0;
-  Tile tile_next = Tile{0, 0, 0};
-  bool more = false;                                      // this lane has a chunk in the span
-  auto fetch = [&]() {
-    fl_next = 0;
-    more = (unsigned)lane < span && c_next < chunks;
-    if (more) {
-      const unsigned t = c_next / kTileChunks;
-      fl_next = p.deferred[c_next];
-      wl_next = t / tpw;
-      tile_next = p.tiles[t - wl_next * tpw];
-    }
-  };
-  fetch();
-  while (__any_sync(0xffffffffu, more)) {
-    const unsigned fl = fl_next, wl = wl_next;
-    const long long elem = tile_next.off + (int)(c_next & (kTileChunks - 1)) * kChunkElems;
-    unsigned sb = 0;                                      // asked for now, looked at after the first rows' loads
-    if (fl != 0u) sb = p.scale_bits[(long long)(p.worker_begin + (int)wl) * p.S + tile_next.seg];
-    c_next += warps * span;
-    fetch();
-    unsigned pending = __ballot_sync(0xffffffffu, fl != 0u);
-    unsigned rows = 0;                                    // flagged rows left of the chunk of lane `cur`
-    int cur = 0;
-    while (pending | rows) {
-      long long row_elem[kBatch];
-      int row_w[kBatch], src[kBatch];
-      bool have[kBatch];
-#pragma unroll
-      for (int a = 0; a < kBatch; ++a) {
-        if (rows == 0u && pending != 0u) {
-          cur = __ffs((int)pending) - 1;
-          pending &= pending - 1u;
-          rows = __shfl_sync(0xffffffffu, fl, cur);
-        }
-        have[a] = rows != 0u;                             // warp-uniform
-        if (!have[a]) continue;
-        const int r = __ffs((int)rows) - 1;
-        rows &= rows - 1u;
-        src[a] = cur;
-        row_elem[a] = __shfl_sync(0xffffffffu, elem, cur) + r * 128;
-        row_w[a] = (int)__shfl_sync(0xffffffffu, wl, cur);
-        gv[a] = ld_f4_stream(p.g + (long long)row_w[a] * p.D + row_elem[a] + lane * 4);
-        row_w[a] += p.worker_begin;
-        ev[a] = ld_f4(p.e + (long long)row_w[a] * p.D + row_elem[a] + lane * 4);
-        if constexpr (L2) hw[a] = held_fetch(p, row_elem[a], lane);
-      }
-#pragma unroll
-      for (int a = 0; a < kBatch; ++a) {
-        if (!have[a]) continue;
-        const GradScale gs = grad_scale<MODE>(__uint_as_float(__shfl_sync(0xffffffffu, sb, src[a])), p.k);
-        deferred_row<MODE, L2>(p, gv[a], ev[a], hw[L2 ? a : 0], gs, row_elem[a],
-                               p.e + (long long)row_w[a] * p.D + row_elem[a] + lane * 4,
-                               p.gcodes + (long long)row_w[a] * p.gcode_bytes + row_elem[a] * kBits / 8, lane);
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Worker phase 2: codes = Q_g level indices of u against the finished scale,
-// packed; e <- u - Q_g(u).  U_IN_E: u was left in e's slot by phase 1.
-// Three blocks per SM (at most 80 registers): with one block of 150 registers the
-// general grids ran at 0.35 of the copy rate, with three at 0.73 (measured).  The stochastic
-// operator's kernels keep to 80 registers by themselves and lose by the bound (3 x 10^7 elements,
-// n = 4, a step: 543 us without, 564 with it; 813 and 831 with the moments on the workers).
-// ---------------------------------------------------------------------------
-template <bool U_IN_E, int MODE, bool L2 = false>
-__global__ void __launch_bounds__(kThreads, MODE == G_STOCHASTIC && !L2 ? 1 : 3)
-worker_quantize_kernel(const WorkerParams p) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // Tiles per round of loads, then of arithmetic and stores.  (Two per round when only e is
-  // read, to have as many loads in flight as the two-array form, was measured slower.)
-  constexpr int kPerRound = 1;
-  for (long long t0 = blockIdx.x; t0 < p.total_tiles; t0 += (long long)kPerRound * gridDim.x) {
-    Tile tile[kPerRound];
-    int wl[kPerRound];
-    bool have[kPerRound];
-    float4 gv[kPerRound][kRows], ev[kPerRound][kRows];
-    HeldRaw hw[kPerRound][L2 ? kRows : 1];
-#pragma unroll
-    for (int a = 0; a < kPerRound; ++a) {
-      const long long t = t0 + (long long)a * gridDim.x;
-      have[a] = t < p.total_tiles;
-      if (!have[a]) continue;
-      wl[a] = (int)(t / p.tiles_per_worker);
-      tile[a] = p.tiles[(int)(t - (long long)wl[a] * p.tiles_per_worker)];
-      const float* gp = p.g + (long long)wl[a] * p.D + tile[a].off;
-      const long long so = (long long)(p.worker_begin + wl[a]) * p.D + tile[a].off;
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        const int idx = r * kRowElems + threadIdx.x * 4;
-        if (idx < tile[a].count) {
-          if constexpr (!U_IN_E) gv[a][r] = ld_f4_stream(gp + idx);
-          ev[a][r] = ld_f4(p.e + so + idx);
-          if constexpr (L2 && !U_IN_E)
-            hw[a][r] = held_fetch(p, tile[a].off + r * kRowElems + warp * 128, lane);
-        }
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < kPerRound; ++a) {
-      if (!have[a]) continue;
-      const int w = p.worker_begin + wl[a];
-      const unsigned sb = p.scale_bits[(long long)w * p.S + tile[a].seg];
-      const float s = __uint_as_float(sb);
-      const GradScale gs = grad_scale<MODE>(s, p.k);
-      if (sb >= 0x7f800000u && threadIdx.x == 0) atomicOr(p.status, 1u);
-      const long long so = (long long)w * p.D + tile[a].off;
-      unsigned char* cw = p.gcodes + (long long)w * p.gcode_bytes;
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        const int idx = r * kRowElems + threadIdx.x * 4;
-        if (idx >= tile[a].count) continue;         // warp-uniform: counts are multiples of 128
-        float ee[4] = {ev[a][r].x, ev[a][r].y, ev[a][r].z, ev[a][r].w};
-        float uu[4];
-        if constexpr (U_IN_E) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) uu[c] = ee[c];
-        } else {
-          float gg[4] = {gv[a][r].x, gv[a][r].y, gv[a][r].z, gv[a][r].w};
-          if constexpr (L2) add_l2_term_held(p, tile[a].off + r * kRowElems + warp * 128, lane, hw[a][r], gg);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) uu[c] = __fadd_rn(gg[c], ee[c]);
-        }
-        unsigned code[4];
-        float en[4];
-        if constexpr (MODE == G_STOCHASTIC) {
-          // the four coordinates of this thread are one block of the stream: counter
-          // (element / 4, worker, step), key = seed
-          const unsigned long long block = (unsigned long long)(tile[a].off + idx) >> 2;
-          const uint4 rnd = philox4x32_10(make_uint4((unsigned)block, (unsigned)(block >> 32), (unsigned)w, p.step),
-                                          make_uint2(p.seed_lo, p.seed_hi));
-          code[0] = quantize_stochastic4(uu, gs, rnd, en);   // the lane's byte of four codes
-        } else if constexpr (MODE == G_TERNARY) {
-          code[0] = quantize_ternary4(uu, gs, en);           // the lane's byte of four codes
-        } else if constexpr (MODE == G_FIVE) {
-          code[0] = quantize_five4(uu, gs, en);              // the lane's 12 bits of four codes
-        } else if constexpr (MODE == G_UNIFORM) {
-          code[0] = quantize_uniform4(uu, gs, p.k, p.L, p.bits, en);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) code[c] = quantize_grad<MODE>(uu[c], gs, p.k, p.L, en[c]);
-        }
-        st_f4(p.e + so + idx, make_float4(en[0], en[1], en[2], en[3]));
-        const long long row_elem = tile[a].off + r * kRowElems + warp * 128;
-        void* dst = cw + row_elem * p.bits / 8;
-        if constexpr (MODE == G_TERNARY || MODE == G_STOCHASTIC) {
-          store_row_of_code_bytes(code[0], dst, lane);
-        } else if constexpr (MODE == G_FIVE) {
-          pack_row_store_fields<3>(code[0], dst, lane);
-        } else if constexpr (MODE == G_UNIFORM) {
-          pack_row_store_fields_rt(p.bits, code[0], dst, lane);
-        } else {
-          pack_row_store_rt(p.bits, code[0], code[1], code[2], code[3], dst, lane);
-        }
-      }
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------

@@ -146,8 +146,6 @@ __host__ __device__ inline size_t resident_smem_bytes(int slots, int estages, bo
   return kRHeadBytes + (size_t)slots * kRSlotBytes +
          (size_t)estages * (resident_stage_bytes(worker_moments) + held_bytes);
 }
-// With the l2 term a stage also carries the tile's held weights: b_x bits (x: 32) per element.
-__host__ __device__ constexpr int resident_held_bytes(int kx, int xbits) { return kTileElems / 8 * (kx < 0 ? 32 : xbits); }
 
 // MODE: grid of Q_g; WM: moments on the workers; L2: the l2 term lambda * (held weights) is
 // added to g first (the held weights come with the stage);
@@ -551,7 +549,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
         unsigned code[4];
         float en[4];
         if constexpr (MODE == G_STOCHASTIC) {
-          // the four coordinates of this thread are one block of the stream, see worker_quantize_kernel
+          // the four coordinates of this thread are one block of the stream, see settle_row
           const unsigned long long block = (unsigned long long)(cd.off + q * kRowElems + gt * 4) >> 2;
           const uint4 rnd = philox4x32_10(
               make_uint4((unsigned)block, (unsigned)(block >> 32), (unsigned)cd.worker, p.step),

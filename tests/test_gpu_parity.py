@@ -510,6 +510,37 @@ def test_rows_left_by_the_sweep_where_they_are_few(kg, l2, chunks_per_warp):
     p.close()
 
 
+@pytest.mark.parametrize("kg", [0, 1])
+@pytest.mark.parametrize("l2", [0.0, 5e-4])
+@pytest.mark.parametrize("tiles", [1, 149, 700])
+def test_open_elements_listed_by_the_sweep(kg, l2, tiles):
+    # Rows of 128 with 1 to 6 elements of other levels (up to 4 are listed one by one, more leave the row
+    # to the second kernel), next to one another so that several share a word of codes and three-bit codes
+    # straddle two; magnitudes on both sides of every midpoint; the pair's maximum in its last element, so
+    # that elements listed under a low bound end up at level 0; the last worker with more of them than
+    # a warp's part of the list holds.  Fewer tiles than blocks, a few more, several per block; ragged.
+    import paper_2004_14180_b200 as qb
+    seg = [max(1, tiles // 2) * 4096 + 130 * (tiles > 1), 77, max(0, tiles // 2 - 1) * 4096 + 900]
+    d, n = sum(seg), 2
+    rng = np.random.default_rng(5 + kg + tiles)
+    p = Pair(seg, n, kg, 0, S_MODE, x1=(rng.standard_normal(d) * 0.2).astype(np.float32),
+             options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    p.set_regularization(l2)
+    for t in range(3):
+        g = (rng.standard_normal((n, d)) * 1e-3).astype(np.float32)
+        for w in range(n):
+            rows = np.arange(0, d - 140, 128)
+            rows = rows[rng.random(rows.size) < (0.3, 0.95)[w]]
+            for k in range(6):
+                at = rows[rng.random(rows.size) < 0.6] + 40 + 9 * t
+                at = at + np.where(rng.random(at.size) < 0.7, k, rng.integers(0, 80, at.size))
+                g[w, at] = rng.choice(np.float32([0.2, -0.24, 0.26, -0.49, 0.51, 0.74, -0.76, 1.0]), at.size)
+            g[w, np.cumsum(seg) - 1] = np.float32(-1.0 - 0.5 * t)
+        p.step(g, threads=8, split_workers=t == 1)
+        p.compare_state()
+    p.close()
+
+
 # ---------------------------------------------------------------- l2 term and step-dependent rates
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
