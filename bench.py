@@ -195,14 +195,15 @@ def algorithmic_bytes(kernel: str, w, placement: str, D: int, gbits: int, xbits:
     split_units = pass_model[1] if pass_model and pass_model[0] > 0 else n * D
     # ternary and five-level codes, moments on the server: the sweep writes e and the codes it can
     # settle, the second kernel the others (how many depends on the data); together every array is
-    # touched once, and what is left is read and written again, which is not counted
+    # touched once, and what is left is read again, which is not counted
     if kernel == "sweep":
         return (12.0 + held + gbits / 8.0) * split_units
-    if kernel == "absmax":      # phase 1: read g, e, write u (worker moments: + read and write m, v)
-        per = (12.0 if server_moments else 28.0) + held
+    if kernel == "absmax":      # phase 1: read g, e (worker moments: + read m, v, write m, v, u)
+        per = (8.0 if server_moments else 28.0) + held
         return per * split_units
-    if kernel == "quantize":    # phase 2: read u, write e and the codes
-        return (8.0 + gbits / 8.0) * split_units
+    if kernel == "quantize":    # phase 2: read g, e (or u), write e and the codes
+        per = (12.0 + held if server_moments else 8.0) + gbits / 8.0
+        return per * split_units
     if kernel == "identity":
         per = ((8.0 + 8.0) if server_moments else (16.0 + 16.0)) + held
         return per * n * D

@@ -248,7 +248,7 @@ struct qadam_ctx {
   int64_t last_server_step;     // steps completed by the server
   int64_t workers_done;         // workers compressed for step last_server_step + 1
   int64_t launches;
-  int form_stages[2] = {0, 0}, settle_stages = 0;   // of the streaming passes' rings, form: without and with the l2 term
+  int form_stages[2] = {0, 0}, settle_stages[2] = {0, 0};   // of the streaming passes' rings, without and with the l2 term
   int grid_ident, grid_server, grid_bcast;
   size_t server_smem;
   // persistent pipelined server pass: stages > 0 when in use
@@ -309,20 +309,30 @@ WorkerKernel pick_form(const qadam_ctx* c, bool l2) {
 }
 
 // The second: codes and e' of everything, or of what the sweep left.
-WorkerKernel pick_settle(const qadam_ctx* c) {
-  const bool swept = sweeps(&c->cfg, c->geo.gmode);
+template <int MODE>
+WorkerKernel pick_settle_mode(bool worker_moments, bool l2) {
+  constexpr bool kSwept = MODE == G_TERNARY || MODE == G_FIVE;         // see sweeps()
+  if (worker_moments) return worker_settle_kernel<MODE, false, true, false>;
+  return l2 ? worker_settle_kernel<MODE, kSwept, false, true> : worker_settle_kernel<MODE, kSwept, false, false>;
+}
+WorkerKernel pick_settle(const qadam_ctx* c, bool l2) {
+  const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
   switch (c->geo.gmode) {
-    case G_STOCHASTIC: return worker_settle_kernel<G_STOCHASTIC, false>;
-    case G_TERNARY: return swept ? worker_settle_kernel<G_TERNARY, true> : worker_settle_kernel<G_TERNARY, false>;
-    case G_FIVE:    return swept ? worker_settle_kernel<G_FIVE, true> : worker_settle_kernel<G_FIVE, false>;
-    case G_POW2:    return worker_settle_kernel<G_POW2, false>;
-    default:        return worker_settle_kernel<G_UNIFORM, false>;
+    case G_STOCHASTIC: return pick_settle_mode<G_STOCHASTIC>(w, l2);
+    case G_TERNARY: return pick_settle_mode<G_TERNARY>(w, l2);
+    case G_FIVE:    return pick_settle_mode<G_FIVE>(w, l2);
+    case G_POW2:    return pick_settle_mode<G_POW2>(w, l2);
+    default:        return pick_settle_mode<G_UNIFORM>(w, l2);
   }
 }
 
 // bytes of a stage of the first launch's ring
 int form_bytes(const qadam_ctx* c, bool l2) {
   return form_stage_bytes(c->cfg.placement == QADAM_PLACE_WORKER, l2 ? held_tile_bytes(c->cfg.kx, c->geo.xbits) : 0);
+}
+
+int settle_bytes(const qadam_ctx* c, bool l2) {
+  return settle_stage_bytes(c->cfg.placement == QADAM_PLACE_WORKER, l2 ? held_tile_bytes(c->cfg.kx, c->geo.xbits) : 0);
 }
 
 WorkerKernel pick_identity(const qadam_ctx* c) {
@@ -612,16 +622,15 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
       const int stage = form_bytes(c, l2 != 0);
       c->form_stages[l2] = stream_stages(max_smem, stage);
       if (sweeps(cfg, c->geo.gmode)) c->form_stages[l2] = c->form_stages[l2] / kStreamGroups * kStreamGroups;
-      ok = c->form_stages[l2] >= 1 &&
+      const int settle = settle_bytes(c, l2 != 0);
+      c->settle_stages[l2] = stream_stages(max_smem, settle) / kStreamGroups * kStreamGroups;
+      ok = c->form_stages[l2] >= 1 && c->settle_stages[l2] >= 1 &&
            cuda_ok(cudaFuncSetAttribute(pick_form(c, l2 != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)stream_smem_bytes(c->form_stages[l2], stage)));
+                                        (int)stream_smem_bytes(c->form_stages[l2], stage))) &&
+           cuda_ok(cudaFuncSetAttribute(pick_settle(c, l2 != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)stream_smem_bytes(c->settle_stages[l2], settle)));
     }
-    c->settle_stages = stream_stages(max_smem, kSettleStageBytes) / kStreamGroups * kStreamGroups;
-    if (!ok || c->settle_stages < 1 ||
-        !cuda_ok(cudaFuncSetAttribute(pick_settle(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)stream_smem_bytes(c->settle_stages, kSettleStageBytes)))) {
-      delete c; return QADAM_ERR_CUDA;
-    }
+    if (!ok) { delete c; return QADAM_ERR_CUDA; }
   }
   c->grid_server = resident_grid(sk, c->server_smem, c->sm_count);
   c->grid_bcast = resident_grid(weight_broadcast_kernel, 0, c->sm_count);
@@ -776,8 +785,8 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
     c->launches += 1;
     {
       LaunchTimer lt(c, QADAM_K_QUANTIZE);
-      q.stages = c->settle_stages;
-      pick_settle(c)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, kSettleStageBytes), c->stream>>>(q);
+      q.stages = c->settle_stages[l2];
+      pick_settle(c, l2)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, settle_bytes(c, l2)), c->stream>>>(q);
     }
     if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
     c->launches += 1;

@@ -1,11 +1,13 @@
 // The worker side of pairs too large for the chip: two pipelined passes over memory.
 //
-//   worker_sweep_kernel    moments on the server, ternary and five-level codes: forms u, leaves it in
-//                          e's place and finishes whatever a lower bound of the scale settles
-//   worker_form_kernel     everything else: forms u (with the moments on the workers, after the moment
-//                          updates), leaves it in e's place, folds max |u|
-//   worker_settle_kernel   codes and e' from u, once the scales are final: of every row, or of what the
-//                          sweep left
+//   worker_sweep_kernel    moments on the server, ternary and five-level codes: forms u and finishes
+//                          whatever a lower bound of the scale settles
+//   worker_form_kernel     everything else: folds max |u|; with the moments on the workers u, formed
+//                          after the moment updates, is left in e's place
+//   worker_settle_kernel   codes and e', once the scales are final: of every row, or of what the sweep
+//                          left; u out of e's place, or of g and e again
+// (Leaving u in e's place in every case moves the same bytes, but a first pass that only reads is
+// faster than one that writes: 1.2 x 10^8 dense elements, n = 2, both passes 792 us with u written.)
 //
 // One CTA per SM.  A producer thread brings tiles of 4096 elements into a ring of shared-memory
 // stages with bulk copies that complete on an mbarrier; consumer warps work from the stages and
@@ -35,7 +37,7 @@ constexpr int kTileChunks = kTileElems / kChunkElems; // 8
 // Words of the workspace the two passes count in; zero between launches (a launch's last CTA clears its own,
 // which spares the step a clear).
 struct StreamCounters {
-  unsigned form_tickets, form_left;      // tiles handed out beyond each CTA's first; CTAs that have left
+  unsigned form_tickets, form_left;      // tiles handed out beyond each CTA's first ones; CTAs that have left
   unsigned settle_tickets, settle_left;
   unsigned rows;                         // rows of 128 elements the sweep flagged
 };
@@ -57,16 +59,18 @@ struct StreamSmem {
   // older one.
   unsigned long long known, published;
   StreamHeader hd[kStreamMaxStages];
-  unsigned pair;            // sweep: of the tile issued last, kNoTile: there are no more
+  unsigned pair;            // sweep: of the tile issued last, kNoTile: there are no more; settle pass: rows flagged
   int abort_flag;
 };
 static_assert(sizeof(StreamSmem) <= kStreamHeadBytes, "head of the shared-memory layout");
 
-// A stage: [g][e][m][v][held weights of the l2 term], or u alone in the settle pass
+// A stage: [g][e][m][v][held weights of the l2 term], or u alone in the settle pass after one with m, v
 __host__ __device__ constexpr int form_stage_bytes(bool worker_moments, int held_bytes) {
   return (worker_moments ? 4 : 2) * kTileElems * 4 + held_bytes;
 }
-constexpr int kSettleStageBytes = kTileElems * 4;
+__host__ __device__ constexpr int settle_stage_bytes(bool worker_moments, int held_bytes) {
+  return worker_moments ? kTileElems * 4 : form_stage_bytes(false, held_bytes);
+}
 inline int stream_stages(int max_smem, int stage_bytes) {
   const int stages = (max_smem - kStreamHeadBytes) / stage_bytes;
   return stages < kStreamMaxStages ? stages : kStreamMaxStages;
@@ -87,16 +91,12 @@ __device__ __forceinline__ void stream_init(StreamSmem* ps, int stages, int read
   __syncthreads();
 }
 
-// The last CTA to leave clears the launch's counters for the next.
+// By the producer thread, once its draws are done: the last CTA's clears the launch's counters for the next.
 __device__ __forceinline__ void stream_leave(unsigned* tickets, unsigned* left, unsigned* also) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(left, 1u) == gridDim.x - 1u) {
-      *tickets = 0u;
-      *left = 0u;
-      if (also) *also = 0u;
-    }
+  if (atomicAdd(left, 1u) == gridDim.x - 1u) {
+    *tickets = 0u;
+    *left = 0u;
+    if (also) *also = 0u;
   }
 }
 
@@ -111,7 +111,8 @@ __device__ __forceinline__ void produce_tiles(const WorkerParams& p, StreamSmem*
   const unsigned total = (unsigned)p.total_tiles, tpw = (unsigned)p.tiles_per_worker;
   int s = 0;
   unsigned ph = 0, armed = 0, armed_par = 0;
-  const auto draw = [&]() { return gridDim.x + atomicAdd(tickets, 1u); };
+  constexpr int kAhead = 8;
+  const auto draw = [&]() { return kAhead * gridDim.x + atomicAdd(tickets, 1u); };
   const auto place = [&](unsigned at) { return backwards ? total - 1u - at : at; };
   const auto descriptor = [&](unsigned at) { return at < total ? p.tiles[place(at) % tpw] : Tile{0, 0, 0}; };
   const auto looked = [&](unsigned at) { return at < total ? look(place(at)) : 0ull; };
@@ -119,24 +120,28 @@ __device__ __forceinline__ void produce_tiles(const WorkerParams& p, StreamSmem*
   const auto stage_free = [&]() {
     return mbar_wait_bounded(&ps->empty[s], ph ^ 1u, abort_flag, p.status, p.spin_limit);
   };
-  // Slot k holds the tile being issued, k + 1 the next, whose descriptor is there, k + 2 one whose
-  // descriptor is asked for now, k + 3 a number on its way: a trip to L2 takes about as long as a tile.
-  // Slots are named by unrolling, not moved along: a move would wait for what is on its way.
-  unsigned nt[4] = {blockIdx.x, draw(), draw(), draw()};
+  // Numbers are drawn kAhead tiles before their turn (the first kAhead are every G-th tile, so that
+  // nothing waits at the start), descriptors asked for two tiles before it: a trip to L2 takes as long as
+  // a tile or two, an atomic on one address for all SMs the longest (drawn three ahead: 1.2 x 10^8
+  // dense elements, n = 2, second pass 388 -> 371 us with eight).  Slots are named by unrolling, not
+  // moved along: a move would wait for what is on its way.
+  unsigned nt[kAhead];
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) nt[k] = blockIdx.x + k * gridDim.x;
   Tile tile[4] = {descriptor(nt[0]), descriptor(nt[1]), {0, 0, 0}, {0, 0, 0}};
   unsigned long long seen[4] = {looked(nt[0]), looked(nt[1]), 0ull, 0ull};
   bool more = true;
   while (more) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      tile[(k + 2) & 3] = descriptor(nt[(k + 2) & 3]);
-      seen[(k + 2) & 3] = looked(nt[(k + 2) & 3]);
+    for (int k = 0; k < kAhead; ++k) {
+      tile[(k + 2) & 3] = descriptor(nt[(k + 2) % kAhead]);
+      seen[(k + 2) & 3] = looked(nt[(k + 2) % kAhead]);
       if (nt[k] >= total || !stage_free()) {
         more = false;
         break;
       }
       const unsigned at = place(nt[k]);
-      if (issue(tile[k], at / tpw, at, seen[k], s, &ps->hd[s])) {
+      if (issue(tile[k & 3], at / tpw, at, seen[k & 3], s, &ps->hd[s])) {
         armed |= 1u << s;
         armed_par = (armed_par & ~(1u << s)) | (ph << s);
         if (++s == stages) { s = 0; ph ^= 1u; }
@@ -150,6 +155,11 @@ __device__ __forceinline__ void produce_tiles(const WorkerParams& p, StreamSmem*
     if (++s == stages) { s = 0; ph ^= 1u; }
   }
   *reinterpret_cast<volatile unsigned*>(&ps->pair) = kNoTile;
+  // (every draw has come back before this CTA counts as gone)
+  unsigned drawn = 0;
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) drawn |= nt[k];
+  if (drawn != kNoTile) __threadfence_block();
   // drain after an abort: nothing may still be landing in shared memory when the CTA exits
   if (*abort_flag) {
     for (int ds = 0; ds < stages; ++ds) {
@@ -199,8 +209,8 @@ __device__ __forceinline__ void fill_header(const WorkerParams& p, StreamHeader*
 // finished in the sweep: 12 + b/8 bytes per element, the least there is.  Of a row with few open
 // elements (at most kListedPerRow) level 0 is written for all, and the open ones are listed with their u:
 // when the scale is known the settle pass goes over the list and mends those whose level turns out not
-// to be 0 (a 4-byte store of e' and an exclusive-or of the code each).  Every other row is flagged, and the
-// settle pass takes its u from e's place: 20 + b/8 bytes in all, as in two full passes.  The error
+// to be 0 (a 4-byte store of e' and an exclusive-or of the code each).  Every other row is left untouched
+// and flagged, and the settle pass reads its g and e again: 20 + b/8 bytes in all, as in two full passes.  The error
 // feedback keeps the codes of heavy-tailed gradients
 // sparse (2^28 elements of the benchmark's mixture after 18 steps: 10 % of the rows hold a code
 // other than level 0, as a rule one or two).  Flagging all of these, the second pass took 1.53 ms there
@@ -233,7 +243,7 @@ worker_sweep_kernel(const WorkerParams p) {
   stream_init(ps, stages, kStreamWarps / kStreamGroups, (unsigned)p.worker_begin * (unsigned)p.S);
 
   if (warp == kStreamWarps) {
-    if (lane == 0)
+    if (lane == 0) {
       produce_tiles(
           p, ps, &p.counters->form_tickets, false, kStreamGroups, [&](unsigned) { return 0ull; },
           [&](const Tile& tile, unsigned wl, unsigned t, unsigned long long, int s, StreamHeader* hd) {
@@ -242,6 +252,8 @@ worker_sweep_kernel(const WorkerParams p) {
             issue_inputs<false, L2>(p, ring + (size_t)s * stage_bytes, tile, wl, &ps->full[s]);
             return true;
           });
+      stream_leave(&p.counters->form_tickets, &p.counters->form_left, nullptr);
+    }
   } else if (warp == kStreamWarps + 1) {
     // ------------------------------------------------------------------ exchange of bounds
     // (ends when the producer has issued its last tile, which its bounded waits see to)
@@ -331,9 +343,11 @@ worker_sweep_kernel(const WorkerParams p) {
 #pragma unroll
       for (int r = 0; r < kChunkRows; ++r) {
         if (first + r * 128 >= hd.count) continue;
-        st_f4(ep + r * 128, u4[r]);
         const unsigned lanes = __ballot_sync(0xffffffffu, row_max[r] > thr);
-        if (lanes == 0u) continue;
+        if (lanes == 0u) {
+          st_f4(ep + r * 128, u4[r]);
+          continue;
+        }
         const float uu[4] = {u4[r].x, u4[r].y, u4[r].z, u4[r].w};
         unsigned open[4], count = kListedPerRow + 1u;
         if (__popc(lanes) <= kListedPerRow) {
@@ -348,6 +362,7 @@ worker_sweep_kernel(const WorkerParams p) {
           flags |= 1u << r;
           continue;
         }
+        st_f4(ep + r * 128, u4[r]);
         unsigned at = listed + 1u;
         listed += count;
 #pragma unroll
@@ -373,12 +388,11 @@ worker_sweep_kernel(const WorkerParams p) {
     if (lane == 0 && flagged) atomicAdd(&p.counters->rows, flagged);
     if (lane == 0 && p.open_stride != 0u) list[0] = listed;
   }
-  stream_leave(&p.counters->form_tickets, &p.counters->form_left, nullptr);
 }
 
 // ---------------------------------------------------------------------------
-// Everything the sweep does not serve: u into e's place (with the moments on the workers after the moment
-// updates of Algorithm 3), max |u| of every (worker, segment) pair.  The maximum is taken on the bit
+// Everything the sweep does not serve: max |u| of every (worker, segment) pair; with the moments on the
+// workers the moment updates of Algorithm 3, and u into e's place.  The maximum is taken on the bit
 // patterns of |u| (monotone for non-negative floats, exact, order-free; a NaN or Inf ends up as the
 // maximum and is reported by the settle pass).  All 16 warps work on one tile: rows row0, row0 + 2
 // of 1024 elements.
@@ -396,7 +410,7 @@ worker_form_kernel(const WorkerParams p) {
   stream_init(ps, stages, kStreamWarps, 0u);
 
   if (warp == kStreamWarps) {
-    if (lane == 0)
+    if (lane == 0) {
       produce_tiles(
           p, ps, &p.counters->form_tickets, false, 1, [&](unsigned) { return 0ull; },
           [&](const Tile& tile, unsigned wl, unsigned t, unsigned long long, int s, StreamHeader* hd) {
@@ -404,6 +418,8 @@ worker_form_kernel(const WorkerParams p) {
             issue_inputs<WM, L2>(p, ring + (size_t)s * stage_bytes, tile, wl, &ps->full[s]);
             return true;
           });
+      stream_leave(&p.counters->form_tickets, &p.counters->form_left, nullptr);
+    }
   } else if (warp < kStreamWarps) {
     const int gt = threadIdx.x & (kThreads - 1), row0 = threadIdx.x / kThreads;
     unsigned mx = 0, cur_pair = ~0u;
@@ -466,14 +482,13 @@ worker_form_kernel(const WorkerParams p) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) uu[c] = __fadd_rn(gg[c], ee[c]);
         }
-        st_f4(p.e + so + q, make_float4(uu[0], uu[1], uu[2], uu[3]));
+        if constexpr (WM) st_f4(p.e + so + q, make_float4(uu[0], uu[1], uu[2], uu[3]));
 #pragma unroll
         for (int c = 0; c < 4; ++c) mx = max(mx, __float_as_uint(fabsf(uu[c])));
       }
     }
     if (cur_pair != ~0u) leave();
   }
-  stream_leave(&p.counters->form_tickets, &p.counters->form_left, nullptr);
 }
 
 // The open elements the sweep listed, now that their scales are final: the code of a listed element
@@ -564,13 +579,13 @@ __device__ __forceinline__ void settle_row(const WorkerParams& p, const float4& 
 }
 
 // The few rows a sweep has flagged: a warp takes 32 chunks (4 tiles) at a time, one byte of flags per
-// lane, and settles their rows eight at a time, so that it keeps as many loads in flight as with full
+// lane, and settles their rows four at a time, so that it keeps as many loads in flight as with full
 // tiles; the flags and descriptors of its next 32 are fetched meanwhile.  Where 32 chunks each would
 // leave warps without any, a warp takes 16, 8, ... 1 (7 x 10^6 elements, n = 1, a third of the rows
 // left: 28 -> 16 us).
-template <int MODE>
+template <int MODE, bool L2>
 __device__ __forceinline__ void settle_few(const WorkerParams& p) {
-  constexpr int kBatch = 8;
+  constexpr int kBatch = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned total = (unsigned)p.total_tiles, tpw = (unsigned)p.tiles_per_worker;
   const unsigned warps = gridDim.x * kStreamWarps, chunks = total * kTileChunks;   // below 2^32: 512 elements each
@@ -602,7 +617,7 @@ __device__ __forceinline__ void settle_few(const WorkerParams& p) {
     unsigned rows = 0;                                    // flagged rows left of the chunk of lane `cur`
     int cur = 0;
     while (pending | rows) {
-      float4 uv[kBatch];
+      float4 gv[kBatch], ev[kBatch];
       long long at[kBatch];
       int row_w[kBatch], src[kBatch];
       bool have[kBatch];
@@ -619,27 +634,33 @@ __device__ __forceinline__ void settle_few(const WorkerParams& p) {
         rows &= rows - 1u;
         src[a] = cur;
         at[a] = __shfl_sync(0xffffffffu, elem, cur) + r * 128 + lane * 4;
-        row_w[a] = p.worker_begin + (int)__shfl_sync(0xffffffffu, wl, cur);
-        uv[a] = ld_f4(p.e + (long long)row_w[a] * p.D + at[a]);
+        row_w[a] = (int)__shfl_sync(0xffffffffu, wl, cur);
+        gv[a] = ld_f4_stream(p.g + (long long)row_w[a] * p.D + at[a]);
+        row_w[a] += p.worker_begin;
+        ev[a] = ld_f4(p.e + (long long)row_w[a] * p.D + at[a]);
       }
 #pragma unroll
       for (int a = 0; a < kBatch; ++a) {
         if (!have[a]) continue;
         const GradScale gs = grad_scale<MODE>(__uint_as_float(__shfl_sync(0xffffffffu, sb, src[a])), p.k);
-        settle_row<MODE>(p, uv[a], gs, row_w[a], at[a], lane);
+        float gg[4] = {gv[a].x, gv[a].y, gv[a].z, gv[a].w};
+        if constexpr (L2) add_l2_term(p, at[a] - lane * 4, lane, gg);
+        settle_row<MODE>(p, make_float4(__fadd_rn(gg[0], ev[a].x), __fadd_rn(gg[1], ev[a].y), __fadd_rn(gg[2], ev[a].z),
+                                        __fadd_rn(gg[3], ev[a].w)), gs, row_w[a], at[a], lane);
       }
     }
   }
 }
 
 // ---------------------------------------------------------------------------
-// Codes and e' from u in e's place.  SWEPT: of the elements the sweep listed and the rows it flagged,
+// Codes and e'.  SWEPT: of the elements the sweep listed and the rows it flagged,
 // the latter tile by tile where they are half of all rows or more, else row by row.  Tiles are gone
 // through from the last to the first: the u written last is still in L2.
 // ---------------------------------------------------------------------------
-template <int MODE, bool SWEPT>
+template <int MODE, bool SWEPT, bool WM, bool L2>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 worker_settle_kernel(const WorkerParams p) {
+  static_assert(!WM || (!SWEPT && !L2), "with the moments on the workers u is in e's place");
   static_assert(!SWEPT || MODE == G_TERNARY || MODE == G_FIVE, "grids the sweep serves");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamSmem* ps = reinterpret_cast<StreamSmem*>(smem_raw);
@@ -647,14 +668,17 @@ worker_settle_kernel(const WorkerParams p) {
   const int stages = p.stages;
   unsigned char* ring = smem_raw + kStreamHeadBytes;
   volatile int* abort_flag = &ps->abort_flag;
-  const unsigned left = SWEPT ? __ldcg(&p.counters->rows) : 0u;
+  // (the count of rows goes through shared memory: read by every CTA before any of them can clear it)
+  stream_init(ps, stages, kStreamWarps / kStreamGroups, SWEPT && threadIdx.x == 0 ? __ldcg(&p.counters->rows) : 0u);
+  const unsigned left = *reinterpret_cast<volatile unsigned*>(&ps->pair);
   const bool tiles = !SWEPT || left / 16u >= (unsigned)p.total_tiles;
-  stream_init(ps, stages, kStreamWarps / kStreamGroups, 0u);
+  const int stage_bytes = settle_stage_bytes(WM, L2 ? held_tile_bytes(p.kx, p.xbits) : 0);
+  __syncthreads();
 
   if (warp == kStreamWarps) {
     unsigned scale_bits = 0u, scale_pair = ~0u;         // read where the pair changes
-    if (lane == 0 && tiles)
-      produce_tiles(
+    if (lane == 0) {
+      if (tiles) produce_tiles(
           p, ps, &p.counters->settle_tickets, true, kStreamGroups,
           [&](unsigned t) { return SWEPT ? reinterpret_cast<const unsigned long long*>(p.deferred)[t] : ~0ull; },
           [&](const Tile& tile, unsigned wl, unsigned t, unsigned long long flags, int s, StreamHeader* hd) {
@@ -666,16 +690,22 @@ worker_settle_kernel(const WorkerParams p) {
             }
             hd->scale_bits = scale_bits;
             hd->flags = flags;
-            const unsigned bytes = (unsigned)tile.count * 4u;
-            mbar_arrive_expect_tx(&ps->full[s], bytes);
-            bulk_load(ring + (size_t)s * kSettleStageBytes, p.e + (long long)hd->worker * p.D + tile.off, bytes,
-                      &ps->full[s]);
+            unsigned char* st = ring + (size_t)s * stage_bytes;
+            if constexpr (WM) {
+              const unsigned bytes = (unsigned)tile.count * 4u;
+              mbar_arrive_expect_tx(&ps->full[s], bytes);
+              bulk_load(st, p.e + (long long)hd->worker * p.D + tile.off, bytes, &ps->full[s]);
+            } else {
+              issue_inputs<false, L2>(p, st, tile, wl, &ps->full[s]);
+            }
             return true;
           });
+      stream_leave(&p.counters->settle_tickets, &p.counters->settle_left, SWEPT ? &p.counters->rows : nullptr);
+    }
   } else if (warp < kStreamWarps) {
     if constexpr (SWEPT) {
       if (p.open_stride != 0u) close_listed<MODE>(p);
-      if (!tiles && left != 0u) settle_few<MODE>(p);
+      if (!tiles && left != 0u) settle_few<MODE, L2>(p);
     }
     const int gt = threadIdx.x & (kThreads - 1);
     int s = threadIdx.x / kThreads;                                 // group g takes stages g, g + groups, ...
@@ -684,10 +714,19 @@ worker_settle_kernel(const WorkerParams p) {
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&ps->full[s], ph, abort_flag, p.status, p.spin_limit))) break;
       const StreamHeader hd = ps->hd[s];
       if (hd.t == kNoTile) break;
-      const float* su = reinterpret_cast<const float*>(ring + (size_t)s * kSettleStageBytes) + gt * 4;
+      const unsigned char* st = ring + (size_t)s * stage_bytes;
+      const float* su = reinterpret_cast<const float*>(st) + gt * 4;
       float4 u4[kRows];
 #pragma unroll
-      for (int r = 0; r < kRows; ++r) u4[r] = *reinterpret_cast<const float4*>(su + r * kRowElems);
+      for (int r = 0; r < kRows; ++r) {
+        u4[r] = *reinterpret_cast<const float4*>(su + r * kRowElems);
+        if constexpr (!WM) {
+          const float4 e4 = *reinterpret_cast<const float4*>(su + kTileElems + r * kRowElems);
+          float gg[4] = {u4[r].x, u4[r].y, u4[r].z, u4[r].w};
+          if constexpr (L2) add_l2_term_staged(p, st + form_stage_bytes(false, 0), r * kRowElems + (gt >> 5) * 128, lane, gg);
+          u4[r] = make_float4(__fadd_rn(gg[0], e4.x), __fadd_rn(gg[1], e4.y), __fadd_rn(gg[2], e4.z), __fadd_rn(gg[3], e4.w));
+        }
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&ps->empty[s]);
       if ((s += kStreamGroups) >= stages) { s -= stages; ph ^= 1u; }
@@ -703,7 +742,6 @@ worker_settle_kernel(const WorkerParams p) {
       }
     }
   }
-  stream_leave(&p.counters->settle_tickets, &p.counters->settle_left, SWEPT ? &p.counters->rows : nullptr);
 }
 
 }  // namespace qadam
