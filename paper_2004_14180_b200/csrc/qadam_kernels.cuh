@@ -128,33 +128,66 @@ __device__ __forceinline__ void add_l2_term(const WorkerParams& p, long long row
 // With the l2 term a pipeline stage also carries its tile's held weights: b_x bits (x: 32) per element.
 __host__ __device__ constexpr int held_tile_bytes(int kx, int xbits) { return kTileElems / 8 * (kx < 0 ? 32 : xbits); }
 
-// The same from a copy of the tile's held weights in shared memory (packed codes, or x itself);
+// The same from a copy of the tile's held weights in shared memory (packed codes, or x itself).  What a
+// thread needs for it is prepared once: a pair of codes moves into the mantissas of two floats whose
+// exponents give them the weight 1; less 2^E + 2^kx these are the weights in grid steps, exactly, and
+// lambda times the step, exact too, times that is fl(lambda w): the same product, rounded once.
+// 3 instructions per element where the fields were shifted, masked, converted and scaled one by one (7).
+struct HeldLane {
+  unsigned m0, m1, g1;     // masks of the two codes, exponent of the second
+  float2 k;                // -(2^E + 2^kx)
+  float unit;              // lambda 2^-(kx+1); 0: one by one (unquantized weights, wide codes, tiny lambda)
+  int word, shift, next;   // the lane's field: first word, bit in it, whether it runs on
+};
+__device__ __forceinline__ HeldLane held_lane(const WorkerParams& p, int lane) {
+  HeldLane h;
+  const int b = p.xbits & 15, bit = 4 * p.xbits * lane;
+  h.unit = p.kx >= 0 && p.xbits <= 8 && p.lambda >= 1e-30f ? __fmul_rn(p.lambda, exp2i(-(p.kx + 1))) : 0.0f;
+  h.m0 = (1u << b) - 1u;
+  h.m1 = h.m0 << b;
+  h.g1 = (unsigned)(150 - b) << 23;
+  const float zero = exp2i(p.kx < 0 ? 0 : p.kx);
+  h.k = make_float2(-(8388608.0f + zero), -(exp2i(23 - b) + zero));
+  h.word = bit >> 5;
+  h.shift = bit & 31;
+  h.next = h.shift + 4 * p.xbits > 32 ? 1 : 0;
+  return h;
+}
 // row: the row's first element in the tile.
-__device__ __forceinline__ void add_l2_term_staged(const WorkerParams& p, const unsigned char* held, int row, int lane,
-                                                   float gg[4]) {
+__device__ __forceinline__ void add_l2_term_staged(const WorkerParams& p, const HeldLane& h, const unsigned char* held,
+                                                   int row, int lane, float gg[4]) {
+  if (h.unit != 0.0f) {
+    const unsigned* words = reinterpret_cast<const unsigned*>(held + row / 8 * p.xbits) + h.word;
+    const unsigned f = __funnelshift_r(words[0], words[h.next], h.shift);
+    const float2 unit = make_float2(h.unit, h.unit);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const unsigned pair = c == 0 ? f : f >> (2 * p.xbits);
+      const float2 w = add2_rn(make_float2(__uint_as_float((pair & h.m0) | 0x4b000000u),
+                                           __uint_as_float((pair & h.m1) | h.g1)), h.k);
+      const float2 term = mul2_rn(w, unit);
+      gg[2 * c] = __fadd_rn(gg[2 * c], term.x);
+      gg[2 * c + 1] = __fadd_rn(gg[2 * c + 1], term.y);
+    }
+    return;
+  }
   float w[4];
   if (p.kx < 0) {
     const float4 v = *reinterpret_cast<const float4*>(held + (row + lane * 4) * 4);
     w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
   } else {
     const unsigned* words = reinterpret_cast<const unsigned*>(held + row / 8 * p.xbits);
-    if (p.xbits <= 8) {
-      const int F = 4 * p.xbits, i = (F * lane) >> 5;
-      const unsigned lo = words[i], hi = ((F * lane) & 31) + F > 32 ? words[i + 1] : 0u;
-      held_decode8(p, lane, lo, hi, w);
-    } else {
-      const int half = 2 * p.xbits;                     // two codes, at most 32 bits
-      const unsigned mask = (1u << p.xbits) - 1u;
-      const float step = exp2i(-(p.kx + 1));
-      const float bias = -(8388608.0f + (float)(1 << p.kx));
+    const int half = 2 * p.xbits;                     // two codes, at most 32 bits
+    const unsigned mask = (1u << p.xbits) - 1u;
+    const float step = exp2i(-(p.kx + 1));
+    const float bias = -(8388608.0f + (float)(1 << p.kx));
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int bit = (2 * lane + h) * half, i = bit >> 5;
-        const unsigned hi = (bit & 31) + half > 32 ? words[i + 1] : 0u;
-        const unsigned f = __funnelshift_r(words[i], hi, bit & 31);
-        w[2 * h] = __fmul_rn(__fadd_rn(__uint_as_float(0x4b000000u | (f & mask)), bias), step);
-        w[2 * h + 1] = __fmul_rn(__fadd_rn(__uint_as_float(0x4b000000u | ((f >> p.xbits) & mask)), bias), step);
-      }
+    for (int i = 0; i < 2; ++i) {
+      const int bit = (2 * lane + i) * half, at = bit >> 5;
+      const unsigned hi = (bit & 31) + half > 32 ? words[at + 1] : 0u;
+      const unsigned f = __funnelshift_r(words[at], hi, bit & 31);
+      w[2 * i] = __fmul_rn(__fadd_rn(__uint_as_float(0x4b000000u | (f & mask)), bias), step);
+      w[2 * i + 1] = __fmul_rn(__fadd_rn(__uint_as_float(0x4b000000u | ((f >> p.xbits) & mask)), bias), step);
     }
   }
 #pragma unroll

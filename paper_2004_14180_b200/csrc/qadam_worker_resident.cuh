@@ -441,6 +441,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
     int s = 0;
     unsigned ph = 0;
     constexpr int kMineL = kRows / kLRowStep;
+    const HeldLane hl = held_lane(p, lane);
     for (long long i = 0; i < my_tiles; ++i) {
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&ps->e_full[s], ph, abort_flag, p.status, spin))) break;
       RLoadHeader* hdp = &ps->load_hd[i & (kRHeaders - 1)];
@@ -469,7 +470,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
           if (q * kRowElems + gt * 4 >= count) continue;               // warp-uniform
           float gg[4] = {g4[r].x, g4[r].y, g4[r].z, g4[r].w};
           float ee[4] = {e4[r].x, e4[r].y, e4[r].z, e4[r].w};
-          if constexpr (L2) add_l2_term_staged(p, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
+          if constexpr (L2) add_l2_term_staged(p, hl, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
           float mm[4] = {m4[r].x, m4[r].y, m4[r].z, m4[r].w};
           float vs[4] = {v4[r].x, v4[r].y, v4[r].z, v4[r].w};
           float uu[4];
@@ -492,7 +493,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
             const float4 g4 = *reinterpret_cast<const float4*>(su + q * kRowElems);
             const float4 e4 = *reinterpret_cast<const float4*>(se + q * kRowElems);
             float gg[4] = {g4.x, g4.y, g4.z, g4.w};
-            if constexpr (L2) add_l2_term_staged(p, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
+            if constexpr (L2) add_l2_term_staged(p, hl, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
             const float4 u4 = make_float4(__fadd_rn(gg[0], e4.x), __fadd_rn(gg[1], e4.y), __fadd_rn(gg[2], e4.z),
                                           __fadd_rn(gg[3], e4.w));
             *reinterpret_cast<float4*>(su + q * kRowElems) = u4;

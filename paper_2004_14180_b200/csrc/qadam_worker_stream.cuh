@@ -276,6 +276,7 @@ worker_sweep_kernel(const WorkerParams p) {
     for (int width = BITS; width < 64; width *= 2) rep |= rep << width;
     constexpr int kRowWords = 4 * BITS;                 // 32-bit words of one row of codes
     const float mid = exp2i(-p.k - 1);                  // the lowest midpoint
+    const HeldLane hl = held_lane(p, lane);
     const int chunk = warp % kTileChunks;               // of the tiles of its group
     const int first = chunk * kChunkElems;
     unsigned run = 0;                                   // maximum of this warp's rows of the pair
@@ -312,7 +313,7 @@ worker_sweep_kernel(const WorkerParams p) {
         const float4 g4 = *reinterpret_cast<const float4*>(sg + r * 128);
         const float4 e4 = *reinterpret_cast<const float4*>(sg + kTileElems + r * 128);
         float gg[4] = {g4.x, g4.y, g4.z, g4.w};
-        if constexpr (L2) add_l2_term_staged(p, st + form_stage_bytes(false, 0), first + r * 128, lane, gg);
+        if constexpr (L2) add_l2_term_staged(p, hl, st + form_stage_bytes(false, 0), first + r * 128, lane, gg);
         u4[r] = make_float4(__fadd_rn(gg[0], e4.x), __fadd_rn(gg[1], e4.y), __fadd_rn(gg[2], e4.z),
                             __fadd_rn(gg[3], e4.w));
         row_max[r] = max(max(__float_as_uint(fabsf(u4[r].x)), __float_as_uint(fabsf(u4[r].y))),
@@ -422,6 +423,7 @@ worker_form_kernel(const WorkerParams p) {
     }
   } else if (warp < kStreamWarps) {
     const int gt = threadIdx.x & (kThreads - 1), row0 = threadIdx.x / kThreads;
+    const HeldLane hl = held_lane(p, lane);
     unsigned mx = 0, cur_pair = ~0u;
     auto leave = [&]() {
       const unsigned r = warp_max(mx);
@@ -453,7 +455,7 @@ worker_form_kernel(const WorkerParams p) {
         }
         if constexpr (L2) {
           float gg[4] = {g4[r].x, g4[r].y, g4[r].z, g4[r].w};
-          add_l2_term_staged(p, st + form_stage_bytes(WM, 0), q + (gt >> 5) * 128, lane, gg);
+          add_l2_term_staged(p, hl, st + form_stage_bytes(WM, 0), q + (gt >> 5) * 128, lane, gg);
           g4[r] = make_float4(gg[0], gg[1], gg[2], gg[3]);
         }
       }
@@ -707,6 +709,7 @@ worker_settle_kernel(const WorkerParams p) {
       if (p.open_stride != 0u) close_listed<MODE>(p);
       if (!tiles && left != 0u) settle_few<MODE, L2>(p);
     }
+    const HeldLane hl = held_lane(p, lane);
     const int gt = threadIdx.x & (kThreads - 1);
     int s = threadIdx.x / kThreads;                                 // group g takes stages g, g + groups, ...
     unsigned ph = 0;
@@ -723,7 +726,7 @@ worker_settle_kernel(const WorkerParams p) {
         if constexpr (!WM) {
           const float4 e4 = *reinterpret_cast<const float4*>(su + kTileElems + r * kRowElems);
           float gg[4] = {u4[r].x, u4[r].y, u4[r].z, u4[r].w};
-          if constexpr (L2) add_l2_term_staged(p, st + form_stage_bytes(false, 0), r * kRowElems + (gt >> 5) * 128, lane, gg);
+          if constexpr (L2) add_l2_term_staged(p, hl, st + form_stage_bytes(false, 0), r * kRowElems + (gt >> 5) * 128, lane, gg);
           u4[r] = make_float4(__fadd_rn(gg[0], e4.x), __fadd_rn(gg[1], e4.y), __fadd_rn(gg[2], e4.z), __fadd_rn(gg[3], e4.w));
         }
       }
