@@ -295,6 +295,14 @@ int resident_grid(K kernel, size_t smem, int sm_count) {
   return std::max(1, per_sm) * sm_count;
 }
 
+// The limit of dynamic shared memory belongs to the kernel, and the call that sets it last holds for all
+// contexts: one that set its own size could take from another's launches what they need.  So every context sets
+// the same, the most the device allows (none of the kernels has static shared memory to leave room for).
+template <typename K>
+bool allow_smem(K kernel, int max_smem) {
+  return cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+}
+
 using WorkerKernel = void (*)(const WorkerParams);
 using ServerKernel = void (*)(const ServerParams);
 
@@ -561,9 +569,10 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     c->d_words = c->geo.words_bytes ? reinterpret_cast<unsigned long long*>(ws + c->geo.off_words) : nullptr;
   }
 
-  int dev = 0;
+  int dev = 0, max_smem = 0;
   if (!cuda_ok(cudaGetDevice(&dev)) ||
-      !cuda_ok(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev))) {
+      !cuda_ok(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev)) ||
+      !cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) {
     delete c; return QADAM_ERR_CUDA;
   }
   c->server_smem = sizeof(float) * (size_t)cfg->n;
@@ -571,17 +580,10 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
     c->server_smem += sizeof(float) * (size_t)cfg->n * ((size_t)1 << c->geo.gbits);
   if (c->server_smem > 200 * 1024) { delete c; return QADAM_ERR_SIZE; }
   ServerKernel sk = pick_server(c);
-  if (c->server_smem > 48 * 1024 &&
-      !cuda_ok(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->server_smem))) {
-    delete c; return QADAM_ERR_CUDA;
-  }
+  if (c->server_smem > 48 * 1024 && !allow_smem(sk, max_smem)) { delete c; return QADAM_ERR_CUDA; }
   // The pipelined server pass needs codes of at most 8 bits, at most kPipeMaxWorkers streams and room
   // for at least two stages in shared memory; otherwise the plain grid-stride kernel runs.
   {
-    int max_smem = 0;
-    if (!cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) {
-      delete c; return QADAM_ERR_CUDA;
-    }
     const bool sm_mom = cfg->placement == QADAM_PLACE_SERVER;
     const bool wide_words = c->geo.gmode == G_POW2 || c->geo.gmode == G_UNIFORM;
     const bool pipe_codes = c->geo.gmode == G_TERNARY || c->geo.gmode == G_STOCHASTIC || c->geo.gmode == G_FIVE ||
@@ -608,27 +610,18 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
                               c->geo.gbits, wide_words, tile_elems)) {
       c->pipe_stages = stages;
       c->pipe_smem = head + (size_t)stages * sb;
-      if (!cuda_ok(cudaFuncSetAttribute(pick_pipe(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)c->pipe_smem))) {
-        delete c; return QADAM_ERR_CUDA;
-      }
+      if (!allow_smem(pick_pipe(c), max_smem)) { delete c; return QADAM_ERR_CUDA; }
     }
   }
   if (!plan_identity_grid(c)) { delete c; return QADAM_ERR_CUDA; }
   if (c->geo.gmode != G_IDENTITY) {
-    int max_smem = 0;
-    bool ok = cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    bool ok = true;
     for (int l2 = 0; l2 < 2 && ok; ++l2) {
-      const int stage = form_bytes(c, l2 != 0);
-      c->form_stages[l2] = stream_stages(max_smem, stage);
+      c->form_stages[l2] = stream_stages(max_smem, form_bytes(c, l2 != 0));
       if (sweeps(cfg, c->geo.gmode)) c->form_stages[l2] = c->form_stages[l2] / kStreamGroups * kStreamGroups;
-      const int settle = settle_bytes(c, l2 != 0);
-      c->settle_stages[l2] = stream_stages(max_smem, settle) / kStreamGroups * kStreamGroups;
-      ok = c->form_stages[l2] >= 1 && c->settle_stages[l2] >= 1 &&
-           cuda_ok(cudaFuncSetAttribute(pick_form(c, l2 != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)stream_smem_bytes(c->form_stages[l2], stage))) &&
-           cuda_ok(cudaFuncSetAttribute(pick_settle(c, l2 != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)stream_smem_bytes(c->settle_stages[l2], settle)));
+      c->settle_stages[l2] = stream_stages(max_smem, settle_bytes(c, l2 != 0)) / kStreamGroups * kStreamGroups;
+      ok = c->form_stages[l2] >= 1 && c->settle_stages[l2] >= 1 && allow_smem(pick_form(c, l2 != 0), max_smem) &&
+           allow_smem(pick_settle(c, l2 != 0), max_smem);
     }
     if (!ok) { delete c; return QADAM_ERR_CUDA; }
   }
@@ -642,19 +635,18 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
   // every CTA resident at once (its store side waits for other CTAs' load sides): one
   // CTA per SM, launched cooperatively.
   {
-    int coop = 0, max_smem = 0;
+    int coop = 0;
     const bool want_split = o.worker_kernel == QADAM_WORKER_STREAMING;
     const bool wm = cfg->placement == QADAM_PLACE_WORKER;
     const bool eligible = !want_split && c->geo.gmode != G_IDENTITY &&
         (c->geo.gmode != G_STOCHASTIC || stochastic_on_chip(cfg, c->geo.D)) &&
-        cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) && coop &&
-        cuda_ok(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) && coop;
     if (eligible) {
       // the CTA's shared memory: a ring of slots for u and a few stages for e (227 KB: 14 in all)
       const int estages = 2;                  // measured: 12 slots + 2 stages beat 11 + 3 and 10 + 4
       const int held = held_tile_bytes(cfg->kx, c->geo.xbits);
       auto slots_for = [&](int held_bytes) {
-        return std::min(((int)max_smem - kRHeadBytes - estages * (resident_stage_bytes(wm) + held_bytes)) / kRSlotBytes,
+        return std::min((max_smem - kRHeadBytes - estages * (resident_stage_bytes(wm) + held_bytes)) / kRSlotBytes,
                         kRMaxSlots);
       };
       const int slots = slots_for(0);
@@ -675,7 +667,7 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
           WorkerResidentKernel k = pick_worker_resident(c, variant >= 2, (variant & 1) != 0);
           int per_sm = 0;
           const size_t smem = variant >= 2 ? c->res_smem_l2 : c->res_smem;
-          fits = cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) &&
+          fits = allow_smem(k, max_smem) &&
                  cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kRThreads, smem)) &&
                  per_sm >= 1;
         }
