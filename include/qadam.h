@@ -142,8 +142,9 @@ typedef struct {
  *  wait_polls     bound on the polls of every wait inside the persistent kernels before
  *                 the kernel gives up with QADAM_ST_TIMEOUT; 0: the default (2^22, seconds).
  *  test_missing_tiles  TESTING ONLY.  The persistent worker kernel is told that every pair
- *                 has this many more tiles than it has, so its waits run out: the way to
- *                 see QADAM_ST_TIMEOUT without a fault.  Leave 0. */
+ *                 has this many more tiles than it has, the streaming passes that a stage
+ *                 has one more reader than it has, so their waits run out: the way to see
+ *                 QADAM_ST_TIMEOUT without a fault.  Leave 0. */
 enum { QADAM_SERVER_AUTO = 0, QADAM_SERVER_PLAIN = 1 };
 enum { QADAM_WORKER_AUTO = 0, QADAM_WORKER_STREAMING = 1 };
 enum { QADAM_HANDOVER_AUTO = 0, QADAM_HANDOVER_COUNTERS = 1 };

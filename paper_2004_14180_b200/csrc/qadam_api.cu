@@ -754,6 +754,7 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
   p.open_stride = 0;
   p.open_regions = 0;
   p.stages = 0;
+  p.missing_readers = c->opt.test_missing_tiles != 0 ? 1 : 0;
   p.counters = c->d_counters;
 
   // the two streaming launches over a tile table

@@ -49,6 +49,7 @@ struct WorkerParams {
   unsigned open_stride;         // 0: no list
   unsigned open_regions;
   int stages;                   // of the streaming passes' rings
+  int missing_readers;          // TESTING: 1: a stage waits for a reader that does not exist (test_missing_tiles)
   StreamCounters* counters;
 };
 

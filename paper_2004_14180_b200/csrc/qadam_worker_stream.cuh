@@ -240,7 +240,7 @@ worker_sweep_kernel(const WorkerParams p) {
   unsigned char* ring = smem_raw + kStreamHeadBytes;
   volatile unsigned long long* known = &ps->known;
   volatile int* abort_flag = &ps->abort_flag;
-  stream_init(ps, stages, kStreamWarps / kStreamGroups, (unsigned)p.worker_begin * (unsigned)p.S);
+  stream_init(ps, stages, kStreamWarps / kStreamGroups + p.missing_readers, (unsigned)p.worker_begin * (unsigned)p.S);
 
   if (warp == kStreamWarps) {
     if (lane == 0) {
@@ -408,7 +408,7 @@ worker_form_kernel(const WorkerParams p) {
   const int stage_bytes = form_stage_bytes(WM, L2 ? held_tile_bytes(p.kx, p.xbits) : 0);
   unsigned char* ring = smem_raw + kStreamHeadBytes;
   volatile int* abort_flag = &ps->abort_flag;
-  stream_init(ps, stages, kStreamWarps, 0u);
+  stream_init(ps, stages, kStreamWarps + p.missing_readers, 0u);
 
   if (warp == kStreamWarps) {
     if (lane == 0) {
@@ -602,9 +602,11 @@ __device__ __forceinline__ void settle_few(const WorkerParams& p) {
     more = (unsigned)lane < span && c_next < chunks;
     if (more) {
       const unsigned t = c_next / kTileChunks;
-      fl_next = p.deferred[c_next];
       wl_next = t / tpw;
       tile_next = p.tiles[t - wl_next * tpw];
+      // (only rows the tile has: a sweep that gave up has left bytes of the workspace as they were)
+      const int rows = (tile_next.count >> 7) - (int)(c_next & (kTileChunks - 1)) * kChunkRows;
+      fl_next = p.deferred[c_next] & ((1u << min(max(rows, 0), kChunkRows)) - 1u);
     }
   };
   fetch();
@@ -671,7 +673,8 @@ worker_settle_kernel(const WorkerParams p) {
   unsigned char* ring = smem_raw + kStreamHeadBytes;
   volatile int* abort_flag = &ps->abort_flag;
   // (the count of rows goes through shared memory: read by every CTA before any of them can clear it)
-  stream_init(ps, stages, kStreamWarps / kStreamGroups, SWEPT && threadIdx.x == 0 ? __ldcg(&p.counters->rows) : 0u);
+  stream_init(ps, stages, kStreamWarps / kStreamGroups + p.missing_readers,
+              SWEPT && threadIdx.x == 0 ? __ldcg(&p.counters->rows) : 0u);
   const unsigned left = *reinterpret_cast<volatile unsigned*>(&ps->pair);
   const bool tiles = !SWEPT || left / 16u >= (unsigned)p.total_tiles;
   const int stage_bytes = settle_stage_bytes(WM, L2 ? held_tile_bytes(p.kx, p.xbits) : 0);
