@@ -91,9 +91,13 @@ __device__ __forceinline__ void stream_init(StreamSmem* ps, int stages, int read
   __syncthreads();
 }
 
-// By the producer thread, once its draws are done: the last CTA's clears the launch's counters for the next.
+// By the producer thread, once it draws no more: the last CTA's clears the launch's counters for the next.  Every
+// CTA's draws, and whatever of the counters it has read, come before its count (release), all counts before the
+// clearing (acquire).
 __device__ __forceinline__ void stream_leave(unsigned* tickets, unsigned* left, unsigned* also) {
-  if (atomicAdd(left, 1u) == gridDim.x - 1u) {
+  unsigned gone;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(gone) : "l"(left) : "memory");
+  if (gone == gridDim.x - 1u) {
     *tickets = 0u;
     *left = 0u;
     if (also) *also = 0u;
@@ -155,11 +159,6 @@ __device__ __forceinline__ void produce_tiles(const WorkerParams& p, StreamSmem*
     if (++s == stages) { s = 0; ph ^= 1u; }
   }
   *reinterpret_cast<volatile unsigned*>(&ps->pair) = kNoTile;
-  // (every draw has come back before this CTA counts as gone)
-  unsigned drawn = 0;
-#pragma unroll
-  for (int k = 0; k < kAhead; ++k) drawn |= nt[k];
-  if (drawn != kNoTile) __threadfence_block();
   // drain after an abort: nothing may still be landing in shared memory when the CTA exits
   if (*abort_flag) {
     for (int ds = 0; ds < stages; ++ds) {

@@ -541,6 +541,54 @@ def test_open_elements_listed_by_the_sweep(kg, l2, tiles):
     p.close()
 
 
+@pytest.mark.parametrize("kg,grid,placement", [(0, 0, S_MODE), (1, 0, S_MODE), (3, 1, S_MODE), (0, 0, W_MODE)])
+def test_streaming_passes_count_anew_in_every_launch(kg, grid, placement):
+    # The tiles of a pass are handed out by a counter beyond each block's first eight, and the pass's last block
+    # sets it back: calls for all and for some of the workers in a row, then replays of a captured step, which
+    # the host cannot help.  More than eight tiles per block; gradients that leave listed elements and rows.
+    import oracle
+    import paper_2004_14180_b200 as qb
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    seg, n = [sms * 3 * 4096 + 300, 5000, 64, sms * 4096 // 2 + 129], 3
+    d = sum(seg)
+    rng = np.random.default_rng(40 + kg)
+    x1 = (rng.standard_normal(d) * 0.2).astype(np.float32)
+    stream = torch.cuda.Stream()
+    q = qb.QAdam(seg, n, kg=kg, kx=0, placement=placement, grid_g=grid, x1=torch.from_numpy(x1), stream=stream,
+                 options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    c = oracle.OracleState(seg, n, kg, 0, placement, 0.9, 0.999, 1e-8, grid_g=grid)
+    c.set_weights(x1)
+    g = c.to_padded((rng.standard_t(3, (n, d)) * 1e-3).astype(np.float32))
+    g_dev = torch.from_numpy(g).cuda()
+
+    def check(scale):
+        torch.cuda.synchronize()
+        c.workers_step(g * np.float32(scale), 1e-3, 8)
+        c.server_step(1e-3)
+        assert np.array_equal(q.gcodes.cpu().numpy(), c.gcodes)
+        for name in ("scales", "x", "m", "v", "e"):
+            assert bits_equal(getattr(q, name).cpu().numpy(), getattr(c, name)), name
+
+    torch.cuda.synchronize()
+    q.step(1, g_dev)
+    check(1.0)
+    for w in range(n):
+        q.worker_compress(2, g_dev[w:w + 1], w, 1)
+    q.server_step(2)
+    check(1.0)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        q.step(3, g_dev)
+    for scale in (1.0, 0.5, 2.0):
+        g_dev.copy_(torch.from_numpy(g * np.float32(scale)))
+        torch.cuda.synchronize()
+        graph.replay()
+        check(scale)
+    assert q.poll_status() == 0
+    del graph
+    q.close()
+
+
 # ---------------------------------------------------------------- l2 term and step-dependent rates
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
