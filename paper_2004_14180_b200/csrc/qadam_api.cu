@@ -304,10 +304,11 @@ bool allow_smem(K kernel, int max_smem) {
 }
 
 using WorkerKernel = void (*)(const WorkerParams);
+using StreamKernel = void (*)(const StreamParams);
 using ServerKernel = void (*)(const ServerParams);
 
 // The first of the two streaming launches: the sweep that settles what it can, or u and its maxima alone.
-WorkerKernel pick_form(const qadam_ctx* c, bool l2) {
+StreamKernel pick_form(const qadam_ctx* c, bool l2) {
   if (sweeps(&c->cfg, c->geo.gmode)) {
     if (c->geo.gmode == G_TERNARY) return l2 ? worker_sweep_kernel<2, true> : worker_sweep_kernel<2, false>;
     return l2 ? worker_sweep_kernel<3, true> : worker_sweep_kernel<3, false>;
@@ -318,12 +319,12 @@ WorkerKernel pick_form(const qadam_ctx* c, bool l2) {
 
 // The second: codes and e' of everything, or of what the sweep left.
 template <int MODE>
-WorkerKernel pick_settle_mode(bool worker_moments, bool l2) {
+StreamKernel pick_settle_mode(bool worker_moments, bool l2) {
   constexpr bool kSwept = MODE == G_TERNARY || MODE == G_FIVE;         // see sweeps()
   if (worker_moments) return worker_settle_kernel<MODE, false, true, false>;
   return l2 ? worker_settle_kernel<MODE, kSwept, false, true> : worker_settle_kernel<MODE, kSwept, false, false>;
 }
-WorkerKernel pick_settle(const qadam_ctx* c, bool l2) {
+StreamKernel pick_settle(const qadam_ctx* c, bool l2) {
   const bool w = c->cfg.placement == QADAM_PLACE_WORKER;
   switch (c->geo.gmode) {
     case G_STOCHASTIC: return pick_settle_mode<G_STOCHASTIC>(w, l2);
@@ -749,17 +750,18 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
   p.seed_lo = (unsigned)c->cfg.seed;
   p.seed_hi = (unsigned)(c->cfg.seed >> 32);
   p.step = (unsigned)step;
-  p.deferred = c->d_deferred;
-  p.open_list = c->d_open;
-  p.open_stride = 0;
-  p.open_regions = 0;
-  p.stages = 0;
-  p.missing_readers = c->opt.test_missing_tiles != 0 ? 1 : 0;
-  p.counters = c->d_counters;
 
   // the two streaming launches over a tile table
   auto streaming = [&](const Tile* tiles, int tiles_per_worker) -> int {
-    WorkerParams q = p;
+    StreamParams q;
+    static_cast<WorkerParams&>(q) = p;
+    q.deferred = c->d_deferred;
+    q.open_list = c->d_open;
+    q.open_stride = 0;
+    q.open_regions = 0;
+    q.stages = 0;
+    q.missing_readers = c->opt.test_missing_tiles != 0 ? 1 : 0;
+    q.counters = c->d_counters;
     q.tiles = tiles;
     q.tiles_per_worker = tiles_per_worker;
     q.total_tiles = (long long)worker_count * tiles_per_worker;

@@ -108,7 +108,7 @@ __device__ __forceinline__ void stream_leave(unsigned* tickets, unsigned* left, 
 // issued (both are asked for two rounds ahead); issue(tile, worker, t, look, stage, header): header and
 // copies of a tile, false if it needs no stage; `ends` marks for the consumers close the ring.
 template <typename Look, typename Issue>
-__device__ __forceinline__ void produce_tiles(const WorkerParams& p, StreamSmem* ps, unsigned* tickets,
+__device__ __forceinline__ void produce_tiles(const StreamParams& p, StreamSmem* ps, unsigned* tickets,
                                               bool backwards, int ends, Look&& look, Issue&& issue) {
   volatile int* abort_flag = &ps->abort_flag;
   const int stages = p.stages;
@@ -230,7 +230,7 @@ constexpr int kListBatch = 4;
 // BITS: code width, 2 (ternary) or 3 (five levels).
 template <int BITS, bool L2>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-worker_sweep_kernel(const WorkerParams p) {
+worker_sweep_kernel(const StreamParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamSmem* ps = reinterpret_cast<StreamSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -399,7 +399,7 @@ worker_sweep_kernel(const WorkerParams p) {
 // ---------------------------------------------------------------------------
 template <bool WM, bool L2>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-worker_form_kernel(const WorkerParams p) {
+worker_form_kernel(const StreamParams p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   StreamSmem* ps = reinterpret_cast<StreamSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -496,7 +496,7 @@ worker_form_kernel(const WorkerParams p) {
 // that has one other than level 0 goes over the level 0 the sweep wrote (as the bits in which the two
 // differ: several elements share a word), and its e' over u.
 template <int MODE>
-__device__ __forceinline__ void close_listed(const WorkerParams& p) {
+__device__ __forceinline__ void close_listed(const StreamParams& p) {
   constexpr int kBits = MODE == G_TERNARY ? 2 : 3;
   const unsigned lane = threadIdx.x & 31, warps = gridDim.x * kStreamWarps;
   const unsigned tpw = (unsigned)p.tiles_per_worker;
@@ -585,7 +585,7 @@ __device__ __forceinline__ void settle_row(const WorkerParams& p, const float4& 
 // leave warps without any, a warp takes 16, 8, ... 1 (7 x 10^6 elements, n = 1, a third of the rows
 // left: 28 -> 16 us).
 template <int MODE, bool L2>
-__device__ __forceinline__ void settle_few(const WorkerParams& p) {
+__device__ __forceinline__ void settle_few(const StreamParams& p) {
   constexpr int kBatch = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned total = (unsigned)p.total_tiles, tpw = (unsigned)p.tiles_per_worker;
@@ -662,7 +662,7 @@ __device__ __forceinline__ void settle_few(const WorkerParams& p) {
 // ---------------------------------------------------------------------------
 template <int MODE, bool SWEPT, bool WM, bool L2>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-worker_settle_kernel(const WorkerParams p) {
+worker_settle_kernel(const StreamParams p) {
   static_assert(!WM || (!SWEPT && !L2), "with the moments on the workers u is in e's place");
   static_assert(!SWEPT || MODE == G_TERNARY || MODE == G_FIVE, "grids the sweep serves");
   extern __shared__ __align__(128) unsigned char smem_raw[];
