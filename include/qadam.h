@@ -130,7 +130,7 @@ typedef struct {
  *                 n <= 64, else the plain grid-stride kernel.  PLAIN: always the latter.
  *  worker_kernel  AUTO: (worker, segment) pairs that fit in the SMs' shared memory go
  *                 through one persistent kernel that reads g and e once; larger pairs take
- *                 two streaming launches (max-abs, then quantize; or a sweep, then the rows it
+ *                 two streaming launches (max-abs, then quantize; or a sweep, then what it
  *                 left), and so do, under the stochastic operator, vectors of fewer than 32
  *                 segments with n * D below 2^23 (and D below 2^20 if the moments are on the
  *                 workers).

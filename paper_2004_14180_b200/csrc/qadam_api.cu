@@ -64,6 +64,14 @@ constexpr int kListTiles = 1024;
 constexpr int64_t kListShare = 64;
 constexpr size_t kListEntries = (size_t)1 << 16;
 
+// Calls of at most this many tiles go through two plain kernels under the stochastic operator in place of the rings,
+// which are one block per SM: few warps for ten Philox rounds per four coordinates, and 2 to 4 us more for the two
+// starts.  Steps, plain / rings, streaming launches only: n = 8, moments on the server, 500 000 elements in all 16.4 us /
+// 18.7, 2 x 10^6 18.5 / 26.6, 8 x 10^6 40.7 / 54.2, 1.6 x 10^7 75.7 / 80.8, 3.2 x 10^7 147 / 141; on the workers
+// 16.7 / 20.2, 24.0 / 28.6, 61.7 / 68.1, 119 / 118, 226 / 219; n = 1 23.8 / 30.2 at 2 x 10^6, 130.5 / 131 at
+// 1.6 x 10^7; with the l2 term, n = 4, 53.6 / 56.5 at 8 x 10^6, 103 / 96 at 1.6 x 10^7.
+constexpr int64_t kPlainTiles = 2048;
+
 struct Geometry {
   std::vector<int64_t> seg_len, seg_off;
   int64_t D = 0;
@@ -134,12 +142,11 @@ bool sweeps(const qadam_config* c, GMode gmode) {
 
 // The stochastic operator on chip, or in two streaming launches.  On chip g and e are read once, but
 // every pair waits for a hand-over between the CTAs, which other pairs or a CTA's next tiles have to
-// cover.  Steps, streaming / on chip (time over time), one segment or eight, moments on the server:
-// n D = 2 x 10^6 0.86 .. 0.95, 4 .. 5 x 10^6 0.92 .. 0.98, 8.4 x 10^6 1.01 .. 1.13, 3.2 x 10^7 1.25 .. 1.32
-// (141 us / 108 at n = 32).  On the workers 8.4 x 10^6 is 1.09 .. 1.10, 3.2 x 10^7 1.30 .. 1.36 (227 us /
-// 169 at n = 32); below that 0.93 .. 1.09 with vectors of 2^20 elements (1.05 in the mean), 0.91 .. 1.17
-// with shorter ones.  64 segments: 0.99 .. 1.4 for either placement from n D = 2 x 10^4 on (33 us / 29
-// at n = 4, 10^6 elements, 200 segments).
+// cover.  Steps, streaming (plain kernels, see kPlainTiles) / on chip, time over time, moments on the server, n = 1, 4, 8:
+// one segment, n D = 2 x 10^6 0.94, 0.83, 1.01, 4.2 x 10^6 0.94, 1.01, 1.05, 8 x 10^6 1.00, 1.01, 1.02; eight segments
+// 0.98, 1.01, 1.01, then 0.99, 1.03, 1.08, then 1.11, 1.03, 1.10; on the workers 0.99 .. 1.13 from 2 x 10^6 on.  Vectors of
+// 2 x 10^4 and 5 x 10^5 would be faster on chip, mostly: 0.93 .. 1.19 in one segment, 1.03 .. 1.39 in eight.  64 segments:
+// 1.3 .. 1.8 for either placement from n D = 2 x 10^4 on (against the rings of the streaming passes).
 bool stochastic_on_chip(const qadam_config* c, int64_t D) {
   return c->num_segments >= 32 || c->n * D >= (int64_t)1 << 23 ||
          (c->placement == QADAM_PLACE_WORKER && D >= (int64_t)1 << 20);
@@ -249,6 +256,7 @@ struct qadam_ctx {
   int64_t workers_done;         // workers compressed for step last_server_step + 1
   int64_t launches;
   int form_stages[2] = {0, 0}, settle_stages[2] = {0, 0};   // of the streaming passes' rings, without and with the l2 term
+  int grid_plain[2][2] = {};    // of the stochastic operator's plain launches: [first, second][without, with the l2 term]
   int grid_ident, grid_server, grid_bcast;
   size_t server_smem;
   // persistent pipelined server pass: stages > 0 when in use
@@ -333,6 +341,17 @@ StreamKernel pick_settle(const qadam_ctx* c, bool l2) {
     case G_POW2:    return pick_settle_mode<G_POW2>(w, l2);
     default:        return pick_settle_mode<G_UNIFORM>(w, l2);
   }
+}
+
+// Both as plain kernels, for small calls under the stochastic operator.
+WorkerKernel pick_absmax(const qadam_ctx* c, bool l2) {
+  if (c->cfg.placement == QADAM_PLACE_WORKER)
+    return l2 ? worker_absmax_kernel<true, true> : worker_absmax_kernel<true, false>;
+  return l2 ? worker_absmax_kernel<false, true> : worker_absmax_kernel<false, false>;
+}
+WorkerKernel pick_toss(const qadam_ctx* c, bool l2) {
+  if (c->cfg.placement == QADAM_PLACE_WORKER) return worker_toss_kernel<true, false>;   // u has the term already
+  return l2 ? worker_toss_kernel<false, true> : worker_toss_kernel<false, false>;
 }
 
 // bytes of a stage of the first launch's ring
@@ -623,6 +642,11 @@ int qadam_create_ex(const qadam_config* cfg, const qadam_buffers* b, const qadam
       c->settle_stages[l2] = stream_stages(max_smem, settle_bytes(c, l2 != 0)) / kStreamGroups * kStreamGroups;
       ok = c->form_stages[l2] >= 1 && c->settle_stages[l2] >= 1 && allow_smem(pick_form(c, l2 != 0), max_smem) &&
            allow_smem(pick_settle(c, l2 != 0), max_smem);
+      if (c->geo.gmode == G_STOCHASTIC) {
+        c->grid_plain[0][l2] = resident_grid(pick_absmax(c, l2 != 0), 0, c->sm_count);
+        c->grid_plain[1][l2] = resident_grid(pick_toss(c, l2 != 0), 0, c->sm_count);
+        ok = ok && c->grid_plain[0][l2] > 0 && c->grid_plain[1][l2] > 0;
+      }
     }
     if (!ok) { delete c; return QADAM_ERR_CUDA; }
   }
@@ -766,6 +790,7 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
     q.tiles_per_worker = tiles_per_worker;
     q.total_tiles = (long long)worker_count * tiles_per_worker;
     const bool l2 = c->lambda != 0.0f;
+    const bool plain = c->geo.gmode == G_STOCHASTIC && q.total_tiles <= kPlainTiles;
     const int grid = (int)std::min<int64_t>(c->sm_count, q.total_tiles);
     if (sweeps(&c->cfg, c->geo.gmode) && q.total_tiles < 1 << 23) {      // (an entry has 23 bits for its tile)
       q.open_regions = (unsigned)grid * kStreamWarps;
@@ -774,14 +799,20 @@ int qadam_worker_compress(qadam_ctx* c, int64_t step, const float* g,
     {
       LaunchTimer lt(c, QADAM_K_ABSMAX);
       q.stages = c->form_stages[l2];
-      pick_form(c, l2)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, form_bytes(c, l2)), c->stream>>>(q);
+      if (plain)
+        pick_absmax(c, l2)<<<(int)std::min<int64_t>(c->grid_plain[0][l2], q.total_tiles), kThreads, 0, c->stream>>>(q);
+      else
+        pick_form(c, l2)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, form_bytes(c, l2)), c->stream>>>(q);
     }
     if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
     c->launches += 1;
     {
       LaunchTimer lt(c, QADAM_K_QUANTIZE);
       q.stages = c->settle_stages[l2];
-      pick_settle(c, l2)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, settle_bytes(c, l2)), c->stream>>>(q);
+      if (plain)
+        pick_toss(c, l2)<<<(int)std::min<int64_t>(c->grid_plain[1][l2], q.total_tiles), kThreads, 0, c->stream>>>(q);
+      else
+        pick_settle(c, l2)<<<grid, kStreamThreads, stream_smem_bytes(q.stages, settle_bytes(c, l2)), c->stream>>>(q);
     }
     if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
     c->launches += 1;

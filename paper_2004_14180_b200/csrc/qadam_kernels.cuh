@@ -131,6 +131,28 @@ __device__ __forceinline__ void add_l2_term(const WorkerParams& p, long long row
   for (int c = 0; c < 4; ++c) gg[c] = __fadd_rn(gg[c], __fmul_rn(p.lambda, w[c]));
 }
 
+// The same in two halves, for kernels that ask for all they need before the first use: codes of at most 8 bits are
+// fetched raw, other weights (and x itself) read where they are added.
+struct HeldRaw {
+  unsigned lo, hi;
+};
+__device__ __forceinline__ HeldRaw held_fetch(const WorkerParams& p, long long row_elem, int lane) {
+  HeldRaw h = {0u, 0u};
+  if (p.kx >= 0 && p.xbits <= 8) held_fetch8(p, row_elem, lane, h.lo, h.hi);
+  return h;
+}
+__device__ __forceinline__ void add_l2_term_fetched(const WorkerParams& p, long long row_elem, int lane,
+                                                    const HeldRaw& h, float gg[4]) {
+  if (p.kx < 0 || p.xbits > 8) {
+    add_l2_term(p, row_elem, lane, gg);
+    return;
+  }
+  float w[4];
+  held_decode8(p, lane, h.lo, h.hi, w);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) gg[c] = __fadd_rn(gg[c], __fmul_rn(p.lambda, w[c]));
+}
+
 // With the l2 term a pipeline stage also carries its tile's held weights: b_x bits (x: 32) per element.
 __host__ __device__ constexpr int held_tile_bytes(int kx, int xbits) { return kTileElems / 8 * (kx < 0 ? 32 : xbits); }
 
@@ -234,6 +256,143 @@ __device__ __forceinline__ float4 ld_f4_stream(const float* p) {
 }
 __device__ __forceinline__ void st_f4(float* p, const float4& v) {
   *reinterpret_cast<float4*>(p) = v;
+}
+
+// CTA-wide max of a 32-bit pattern; result valid in thread 0.
+__device__ __forceinline__ unsigned block_max(unsigned v, unsigned* smem8) {
+  v = warp_max(v);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) smem8[warp] = v;
+  __syncthreads();
+  unsigned r = 0;
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) r = max(r, smem8[w]);
+  }
+  __syncthreads();
+  return r;
+}
+
+// ---------------------------------------------------------------------------
+// The two streaming launches as plain kernels, for calls of few tiles under the stochastic operator (see
+// kPlainTiles; the rings of the streaming passes take their place above).  First max |u| of every (worker, segment)
+// pair; with the moments on the workers the moment updates too, and u into e's place.  The maximum is taken on the bit
+// patterns (exact, order-free).  Internal linkage: this header is included by more than one source file.
+// ---------------------------------------------------------------------------
+template <bool WORKER_MOMENTS, bool L2>
+static __global__ void __launch_bounds__(kThreads, WORKER_MOMENTS ? 2 : (L2 ? 3 : 4))
+worker_absmax_kernel(const WorkerParams p) {
+  __shared__ unsigned red[kThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned mx = 0;
+  long long cur_pair = -1;
+  auto leave = [&]() {
+    const unsigned r = block_max(mx, red);
+    if (threadIdx.x == 0 && r) atomicMax(p.scale_bits + cur_pair, r);
+  };
+  for (long long t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
+    const int wl = (int)(t / p.tiles_per_worker);
+    const Tile tile = p.tiles[(int)(t - (long long)wl * p.tiles_per_worker)];
+    const int w = p.worker_begin + wl;
+    const long long pair = (long long)w * p.S + tile.seg;
+    if (pair != cur_pair) {
+      if (cur_pair >= 0) leave();
+      mx = 0;
+      cur_pair = pair;
+    }
+    const float* gp = p.g + (long long)wl * p.D + tile.off;
+    const long long so = (long long)w * p.D + tile.off;
+    float4 gv[kRows], ev[kRows], mv[kRows], vv[kRows];
+    HeldRaw hw[L2 ? kRows : 1];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int idx = r * kRowElems + threadIdx.x * 4;
+      if (idx >= tile.count) continue;
+      gv[r] = ld_f4_stream(gp + idx);
+      ev[r] = ld_f4(p.e + so + idx);
+      if constexpr (WORKER_MOMENTS) {
+        mv[r] = ld_f4(p.m + so + idx);
+        vv[r] = ld_f4(p.v + so + idx);
+      }
+      if constexpr (L2) hw[r] = held_fetch(p, tile.off + r * kRowElems + warp * 128, lane);
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int idx = r * kRowElems + threadIdx.x * 4;
+      if (idx >= tile.count) continue;
+      float gg[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w};
+      const float ee[4] = {ev[r].x, ev[r].y, ev[r].z, ev[r].w};
+      float uu[4];
+      if constexpr (L2) add_l2_term_fetched(p, tile.off + r * kRowElems + warp * 128, lane, hw[r], gg);
+      if constexpr (WORKER_MOMENTS) {
+        float mm[4] = {mv[r].x, mv[r].y, mv[r].z, mv[r].w};
+        float vs[4] = {vv[r].x, vv[r].y, vv[r].z, vv[r].w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          moments(p.h, gg[c], mm[c], vs[c]);
+          uu[c] = __fadd_rn(adam_step(p.h, mm[c], vs[c], p.alpha), ee[c]);
+        }
+        st_f4(p.m + so + idx, make_float4(mm[0], mm[1], mm[2], mm[3]));
+        st_f4(p.v + so + idx, make_float4(vs[0], vs[1], vs[2], vs[3]));
+        st_f4(p.e + so + idx, make_float4(uu[0], uu[1], uu[2], uu[3]));
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) uu[c] = __fadd_rn(gg[c], ee[c]);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) mx = max(mx, __float_as_uint(fabsf(uu[c])));
+    }
+  }
+  if (cur_pair >= 0) leave();
+}
+
+// Then codes and e' of the stochastic operator; WORKER_MOMENTS: u is in e's place.  The four coordinates of a thread
+// are one block of the stream: counter (element / 4, worker, step), key = seed.  Three blocks per SM: left to itself
+// the compiler takes 97 registers, which are two (8 x 10^6 elements, n = 4: 45.1 us a step against 43.0).
+template <bool WORKER_MOMENTS, bool L2>
+static __global__ void __launch_bounds__(kThreads, 3)
+worker_toss_kernel(const WorkerParams p) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (long long t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
+    const int wl = (int)(t / p.tiles_per_worker);
+    const Tile tile = p.tiles[(int)(t - (long long)wl * p.tiles_per_worker)];
+    const int w = p.worker_begin + wl;
+    const float* gp = p.g + (long long)wl * p.D + tile.off;
+    const long long so = (long long)w * p.D + tile.off;
+    float4 gv[kRows], ev[kRows];
+    HeldRaw hw[L2 ? kRows : 1];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int idx = r * kRowElems + threadIdx.x * 4;
+      if (idx >= tile.count) continue;
+      if constexpr (!WORKER_MOMENTS) gv[r] = ld_f4_stream(gp + idx);
+      ev[r] = ld_f4(p.e + so + idx);
+      if constexpr (L2) hw[r] = held_fetch(p, tile.off + r * kRowElems + warp * 128, lane);
+    }
+    const unsigned sb = p.scale_bits[(long long)w * p.S + tile.seg];
+    const GradScale gs = grad_scale<G_STOCHASTIC>(__uint_as_float(sb), p.k);
+    if (sb >= 0x7f800000u && threadIdx.x == 0) atomicOr(p.status, 1u);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const int idx = r * kRowElems + threadIdx.x * 4;
+      if (idx >= tile.count) continue;                  // warp-uniform: counts are multiples of 128
+      float uu[4] = {ev[r].x, ev[r].y, ev[r].z, ev[r].w};
+      if constexpr (!WORKER_MOMENTS) {
+        float gg[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w};
+        if constexpr (L2) add_l2_term_fetched(p, tile.off + r * kRowElems + warp * 128, lane, hw[r], gg);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) uu[c] = __fadd_rn(gg[c], uu[c]);
+      }
+      const unsigned long long block = (unsigned long long)(tile.off + idx) >> 2;
+      const uint4 rnd = philox4x32_10(make_uint4((unsigned)block, (unsigned)(block >> 32), (unsigned)w, p.step),
+                                      make_uint2(p.seed_lo, p.seed_hi));
+      float en[4];
+      const unsigned code = quantize_stochastic4(uu, gs, rnd, en);      // the lane's byte of four codes
+      st_f4(p.e + so + idx, make_float4(en[0], en[1], en[2], en[3]));
+      store_row_of_code_bytes(code, p.gcodes + (long long)w * p.gcode_bytes +
+                                        (tile.off + r * kRowElems + warp * 128) * p.bits / 8, lane);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------

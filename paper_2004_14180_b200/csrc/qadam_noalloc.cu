@@ -50,63 +50,6 @@ inline bool cuda_ok(cudaError_t e) {
   return true;
 }
 
-// CTA-wide max of a 32-bit pattern; result valid in thread 0.
-__device__ __forceinline__ unsigned block_max(unsigned v, unsigned* smem8) {
-  v = warp_max(v);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) smem8[warp] = v;
-  __syncthreads();
-  unsigned r = 0;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) r = max(r, smem8[w]);
-  }
-  __syncthreads();
-  return r;
-}
-
-// Running max of |g + e| per worker, on the bit patterns (monotone for non-negative floats, exact,
-// order-free); grid-stride over the tile table, one segment per worker.  A plain kernel: the pipelined
-// passes count in a workspace, which this entry point does not have.
-__global__ void __launch_bounds__(kThreads, 4)
-static_absmax_kernel(const WorkerParams p) {
-  __shared__ unsigned red[kThreads / 32];
-  unsigned mx = 0;
-  int cur = -1;
-  auto leave = [&]() {
-    const unsigned r = block_max(mx, red);
-    if (threadIdx.x == 0 && r) atomicMax(p.scale_bits + cur, r);
-  };
-  for (long long t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
-    const int w = (int)(t / p.tiles_per_worker);
-    const Tile tile = p.tiles[(int)(t - (long long)w * p.tiles_per_worker)];
-    if (w != cur) {
-      if (cur >= 0) leave();
-      mx = 0;
-      cur = w;
-    }
-    const long long o = (long long)w * p.D + tile.off;
-    float4 gv[kRows], ev[kRows];
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      const int idx = r * kRowElems + threadIdx.x * 4;
-      if (idx < tile.count) {
-        gv[r] = ld_f4_stream(p.g + o + idx);
-        ev[r] = ld_f4(p.e + o + idx);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      if (r * kRowElems + threadIdx.x * 4 >= tile.count) continue;
-      mx = max(mx, __float_as_uint(fabsf(__fadd_rn(gv[r].x, ev[r].x))));
-      mx = max(mx, __float_as_uint(fabsf(__fadd_rn(gv[r].y, ev[r].y))));
-      mx = max(mx, __float_as_uint(fabsf(__fadd_rn(gv[r].z, ev[r].z))));
-      mx = max(mx, __float_as_uint(fabsf(__fadd_rn(gv[r].w, ev[r].w))));
-    }
-  }
-  if (cur >= 0) leave();
-}
-
 // Address of the scratch and launch width on the current device; looked up once per
 // device, before anything is enqueued.
 int setup_for_current_device(DeviceSetup* out) {
@@ -120,7 +63,7 @@ int setup_for_current_device(DeviceSetup* out) {
     int sms = 0, per_sm = 0;
     if (!cuda_ok(cudaGetSymbolAddress((void**)&ptr, g_static_scratch)) || ptr == nullptr ||
         !cuda_ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
-        !cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, static_absmax_kernel, kThreads, 0)))
+        !cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, worker_absmax_kernel<false, false>, kThreads, 0)))
       return QADAM_ERR_CUDA;
     d.grid = sms * (per_sm > 0 ? per_sm : 1);
     d.scratch = ptr;
@@ -195,7 +138,7 @@ extern "C" int qadam_worker_scales_static(const float* g, const float* e, int64_
 
   long long grid = setup.grid;
   if (grid > p.total_tiles) grid = p.total_tiles;
-  static_absmax_kernel<<<(int)grid, kThreads, 0, st>>>(p);
+  worker_absmax_kernel<false, false><<<(int)grid, kThreads, 0, st>>>(p);
   if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;
   static_copy_scales_kernel<<<(n + 255) / 256, 256, 0, st>>>(acc, scales, n);
   if (!cuda_ok(cudaGetLastError())) return QADAM_ERR_CUDA;

@@ -852,6 +852,27 @@ def test_stochastic_ternary_operator_at_the_ends_of_its_routes(placement, seg, n
     p.close()
 
 
+@pytest.mark.parametrize("placement", [S_MODE, W_MODE])
+@pytest.mark.parametrize("kx", [-1, 3, 14])
+@pytest.mark.parametrize("tiles", [2, 2048, 2049])
+def test_stochastic_ternary_operator_in_either_form_of_the_streaming_launches(placement, kx, tiles):
+    # up to 2048 tiles of a call plain kernels, above it the rings: on both sides of the line, with held weights of
+    # 5 bits (fields that run on into the next word), 16 bits and as they are; ragged ends, calls for some workers
+    import paper_2004_14180_b200 as qb
+    n = 1 if tiles % 2 or tiles == 2 else 2
+    seg = [(tiles // n - 1) * 4096 - 129, 700]
+    assert n * sum(-(-length // 4096) for length in seg) == tiles
+    d = sum(seg)
+    rng = np.random.default_rng(950 + tiles)
+    p = Pair(seg, n, 0, kx, placement, x1=(rng.standard_normal(d) * 0.2).astype(np.float32), grid_g=2, seed=79,
+             options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    for t, lam in enumerate((0.0, 5e-4)):
+        p.set_regularization(lam)
+        p.step(_rand_grads(rng, n, d), threads=8, split_workers=t == 1)
+        p.compare_state()
+    p.close()
+
+
 def test_stochastic_operator_is_ternary_only():
     import paper_2004_14180_b200 as qb
     with pytest.raises(qb.QAdamError) as ei:
