@@ -581,9 +581,11 @@ __device__ __forceinline__ void settle_row(const WorkerParams& p, const float4& 
 
 // The few rows a sweep has flagged: a warp takes 32 chunks (4 tiles) at a time, one byte of flags per
 // lane, and settles their rows four at a time, so that it keeps as many loads in flight as with full
-// tiles; the flags and descriptors of its next 32 are fetched meanwhile.  Where 32 chunks each would
-// leave warps without any, a warp takes 16, 8, ... 1 (7 x 10^6 elements, n = 1, a third of the rows
-// left: 28 -> 16 us).
+// tiles; the flags and descriptors of its next 32 are fetched meanwhile.  The rows left crowd where a pair
+// begins and its bound is low, so a warp takes 16, 8, ... 1 chunks at a time where it would have fewer than eight
+// turns (Student-t gradients, 1.2 x 10^7 elements, n = 4, a fifth of the rows left, this pass: one turn 110 us, four
+// 48, eight 43; hardly a row left: 12.9, 14.6, 16.9).  The held weights of the l2 term are asked for with g and e
+// (the same with the term: one turn 183 us, four 58, eight 52).
 template <int MODE, bool L2>
 __device__ __forceinline__ void settle_few(const StreamParams& p) {
   constexpr int kBatch = 4;
@@ -591,7 +593,7 @@ __device__ __forceinline__ void settle_few(const StreamParams& p) {
   const unsigned total = (unsigned)p.total_tiles, tpw = (unsigned)p.tiles_per_worker;
   const unsigned warps = gridDim.x * kStreamWarps, chunks = total * kTileChunks;   // below 2^32: 512 elements each
   unsigned span = 32u;
-  while (span > 1u && chunks < span * warps) span >>= 1;
+  while (span > 1u && chunks < 8u * span * warps) span >>= 1;
   unsigned c_next = (blockIdx.x * kStreamWarps + warp) * span + (unsigned)lane;
   unsigned fl_next = 0, wl_next = 0;
   Tile tile_next = Tile{0, 0, 0};
@@ -621,6 +623,7 @@ __device__ __forceinline__ void settle_few(const StreamParams& p) {
     int cur = 0;
     while (pending | rows) {
       float4 gv[kBatch], ev[kBatch];
+      HeldRaw hw[L2 ? kBatch : 1];
       long long at[kBatch];
       int row_w[kBatch], src[kBatch];
       bool have[kBatch];
@@ -641,13 +644,14 @@ __device__ __forceinline__ void settle_few(const StreamParams& p) {
         gv[a] = ld_f4_stream(p.g + (long long)row_w[a] * p.D + at[a]);
         row_w[a] += p.worker_begin;
         ev[a] = ld_f4(p.e + (long long)row_w[a] * p.D + at[a]);
+        if constexpr (L2) hw[a] = held_fetch(p, at[a] - lane * 4, lane);
       }
 #pragma unroll
       for (int a = 0; a < kBatch; ++a) {
         if (!have[a]) continue;
         const GradScale gs = grad_scale<MODE>(__uint_as_float(__shfl_sync(0xffffffffu, sb, src[a])), p.k);
         float gg[4] = {gv[a].x, gv[a].y, gv[a].z, gv[a].w};
-        if constexpr (L2) add_l2_term(p, at[a] - lane * 4, lane, gg);
+        if constexpr (L2) add_l2_term_fetched(p, at[a] - lane * 4, lane, hw[a], gg);
         settle_row<MODE>(p, make_float4(__fadd_rn(gg[0], ev[a].x), __fadd_rn(gg[1], ev[a].y), __fadd_rn(gg[2], ev[a].z),
                                         __fadd_rn(gg[3], ev[a].w)), gs, row_w[a], at[a], lane);
       }

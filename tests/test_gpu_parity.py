@@ -511,6 +511,47 @@ def test_rows_left_by_the_sweep_where_they_are_few(kg, l2, chunks_per_warp):
 
 
 @pytest.mark.parametrize("kg", [0, 1])
+@pytest.mark.parametrize("kx,l2", [(0, 0.0), (0, 5e-4), (3, 5e-4), (14, 5e-4), (-1, 5e-4)])
+@pytest.mark.parametrize("chunks_per_warp", [0.4, 3.5, 17, 40])
+def test_rows_of_many_open_elements_where_they_are_few(kg, kx, l2, chunks_per_warp):
+    # Rows with more open elements than the sweep lists (4) are left to the second kernel, which goes row by row
+    # where they are fewer than half: spans of 1, 2 and 4 chunks of 512 elements per warp (the next span's flags are
+    # fetched ahead).  One row in twenty, in places side by side; every chunk holds the pair's maximum, so what is left
+    # does not depend on the order in which the sweep learns it.  Held weights of 2, 5 and 16 bits and as they are.
+    import paper_2004_14180_b200 as qb
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 16
+    n = 2
+    most = int(warps * chunks_per_warp) * 512 // n
+    seg = [most * 6 // 10 + 77, 130, 4096, most * 3 // 10 + 2000, 1, 513, most // 10 + 1]
+    d, tiles = sum(seg), n * sum(-(-length // 4096) for length in seg)
+    rng = np.random.default_rng(63 + kg)
+    p = Pair(seg, n, kg, kx, S_MODE, x1=(rng.standard_normal(d) * 0.2).astype(np.float32),
+             options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    p.set_regularization(l2)
+    for t in range(2 if chunks_per_warp < 10 else 1):
+        g, _ = _gradients_of_few_open_rows(rng, seg, n, t)
+        left = rows = 0
+        for w in range(n):
+            big, a = np.float32(1 + 0.5 * w + 0.25 * t), 0
+            for length in seg:
+                v = g[w, a:a + length]
+                full = np.arange(length // 128)
+                at = full[(rng.random(full.size) < 0.03) | ((full // 8) % 100 == 3)]
+                for k in range(8):
+                    where = at * 128 + rng.integers(0, 128, at.size)
+                    keep = np.abs(v[where]) < big
+                    v[where[keep]] = big * rng.choice(np.float32([0.6, -0.7, 0.8, -0.9]), int(keep.sum()))
+                above = np.add.reduceat(np.abs(v) > big * np.float32(0.5 ** (kg + 1)), np.arange(0, length, 128))
+                left, rows = left + int((above > 4).sum()), rows + above.size
+                a += length
+        if t == 0:
+            assert 0 < left < 16 * tiles and left < 0.5 * rows
+        p.step(g, threads=8, split_workers=t == 1)
+        p.compare_state()
+    p.close()
+
+
+@pytest.mark.parametrize("kg", [0, 1])
 @pytest.mark.parametrize("l2", [0.0, 5e-4])
 @pytest.mark.parametrize("tiles", [1, 149, 700])
 def test_open_elements_listed_by_the_sweep(kg, l2, tiles):
