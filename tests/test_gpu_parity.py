@@ -652,6 +652,30 @@ def test_l2_term(kg, kx, placement):
 
 
 @pytest.mark.parametrize("placement", [S_MODE, W_MODE])
+@pytest.mark.parametrize("kg,grid", [(0, 0), (1, 0), (2, 0), (3, 1)])
+@pytest.mark.parametrize("kx", [-1, 0, 1, 4, 6, 7, 10, 14])
+def test_l2_term_in_streaming_launches(kx, kg, grid, placement):
+    # Held weights of every kind come with the stages of the rings: 2 to 16 bits (fields that run on into the next
+    # word, 8 bits and more than 8), and as they are; several tiles per block, ragged ends.  lambda on both sides of
+    # 1e-30, below which a code is decoded another way, on gradients of zeros in two segments, so that u is the term.
+    import paper_2004_14180_b200 as qb
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    seg, n = [sms * 4096 + 300, 9000, 64, 129, 4096], 2
+    d = sum(seg)
+    rng = np.random.default_rng(310 + 10 * kg + kx)
+    p = Pair(seg, n, kg, kx, placement, x1=(rng.standard_normal(d) * 0.25).astype(np.float32), grid_g=grid,
+             options=qb.QAdamOptions(worker_kernel=qb.WORKER_STREAMING))
+    for t, lam in enumerate((1.1e-30, 9e-31, 0.3, 5e-4)):
+        p.set_regularization(lam)
+        g = _rand_grads(rng, n, d)
+        if t < 2:
+            g[:, sms * 4096:sms * 4096 + 9364] = 0.0
+        p.step(g, threads=8, split_workers=t == 2)
+        p.compare_state()
+    p.close()
+
+
+@pytest.mark.parametrize("placement", [S_MODE, W_MODE])
 def test_step_dependent_rates(placement):
     """Assumption 2: theta_t = 1 - theta/t, alpha_t = alpha/sqrt(t), a decaying beta_t."""
     rng = np.random.default_rng(41)
