@@ -181,10 +181,14 @@ __device__ __forceinline__ HeldLane held_lane(const WorkerParams& p, int lane) {
   h.next = h.shift + 4 * p.xbits > 32 ? 1 : 0;
   return h;
 }
-// row: the row's first element in the tile.
+// row: the row's first element in the tile.  PREPARED = false: field by field in any case, for the on-chip kernel with the
+// moments on the workers, which has no registers for the masks (they made it spill: weights of 16 bits, ResNet-18-shaped
+// set, n = 8, 501 us a step against 496; BERT-shaped set, n = 16, 9.32 ms against 9.22; of at most 8 bits the same).
+// Its five-level kernel keeps the masks (weights of 3 bits 487 us against 491).
+template <bool PREPARED = true>
 __device__ __forceinline__ void add_l2_term_staged(const WorkerParams& p, const HeldLane& h, const unsigned char* held,
                                                    int row, int lane, float gg[4]) {
-  if (h.unit != 0.0f) {
+  if (PREPARED && h.unit != 0.0f) {
     const unsigned* words = reinterpret_cast<const unsigned*>(held + row / 8 * p.xbits) + h.word;
     const unsigned f = __funnelshift_r(words[0], words[h.next], h.shift);
     const float2 unit = make_float2(h.unit, h.unit);
@@ -203,6 +207,10 @@ __device__ __forceinline__ void add_l2_term_staged(const WorkerParams& p, const 
   if (p.kx < 0) {
     const float4 v = *reinterpret_cast<const float4*>(held + (row + lane * 4) * 4);
     w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+  } else if (!PREPARED && p.xbits <= 8) {
+    const unsigned* words = reinterpret_cast<const unsigned*>(held + row / 8 * p.xbits);
+    const int bit = 4 * p.xbits * lane, at = bit >> 5;
+    held_decode8(p, lane, words[at], (bit & 31) + 4 * p.xbits > 32 ? words[at + 1] : 0u, w);
   } else {
     const unsigned* words = reinterpret_cast<const unsigned*>(held + row / 8 * p.xbits);
     const int half = 2 * p.xbits;                     // two codes, at most 32 bits

@@ -470,7 +470,7 @@ worker_resident_kernel(const WorkerResidentParams rp) {
           if (q * kRowElems + gt * 4 >= count) continue;               // warp-uniform
           float gg[4] = {g4[r].x, g4[r].y, g4[r].z, g4[r].w};
           float ee[4] = {e4[r].x, e4[r].y, e4[r].z, e4[r].w};
-          if constexpr (L2) add_l2_term_staged(p, hl, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
+          if constexpr (L2) add_l2_term_staged<!WM || MODE == G_FIVE>(p, hl, held, q * kRowElems + (gt >> 5) * 128, lane, gg);
           float mm[4] = {m4[r].x, m4[r].y, m4[r].z, m4[r].w};
           float vs[4] = {v4[r].x, v4[r].y, v4[r].z, v4[r].w};
           float uu[4];
