@@ -167,7 +167,11 @@ typedef struct {
   void* wcodes;               /* [wcode_bytes] out: packed Q_x(x); may be NULL when kx = -1       */
   float* wresid;              /* [D] out, optional (NULL to skip): x - Q_x(x)                     */
   void* workspace;            /* scratch, workspace_bytes of qadam_query_sizes, 256-byte aligned;
-                                 the library keeps tables here between calls: do not touch it   */
+                                 the library keeps tables here between calls: do not touch it.
+                                 With the moments on the server and ternary or five-level codes
+                                 it holds a byte per 512 gradient elements and a list of 512 KB
+                                 and, of segments of more than 1024 x 4096 elements, an eighth
+                                 of a byte per gradient element (0.5 GB at 16 x 2^28)          */
   size_t workspace_bytes;
   uint32_t* status;           /* one word; qadam_create clears it                                 */
   float* wfeedback;           /* [D] optional (NULL: off; needs kx >= 0), zeros at creation.  An

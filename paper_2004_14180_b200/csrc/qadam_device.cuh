@@ -13,7 +13,7 @@
 namespace qadam {
 
 constexpr int kAlign = 128;        // elements: segment starts, tile starts and tile lengths are multiples
-constexpr int kThreads = 256;      // threads per CTA in every kernel
+constexpr int kThreads = 256;      // threads per CTA of the plain kernels; a group of consumers of the pipelined ones
 constexpr int kRows = 4;           // float4 rows per thread and tile
 constexpr int kRowElems = kThreads * 4;          // 1024 elements per CTA-wide row
 constexpr int kTileElems = kRows * kRowElems;    // 4096 elements per tile
@@ -562,8 +562,9 @@ __device__ __forceinline__ float2 fma2_rn(float2 a, float2 b, float2 c) {
 // second may be brought onto SMs that the first has left once all blocks of the first have
 // said so; it waits here until the first has ended and its writes are visible.
 // Only the on-chip worker kernel, one block per SM, says so (a step 2 .. 4 us shorter).  The
-// streaming kernels do not: with blocks of the server pass coming up between theirs, steps of
-// 6 x 10^7 elements, n = 1, took 441 us against 425, of 1.2 x 10^8, n = 2, 1235 against 1204.
+// streaming kernels do not: plain ones lost by it, with blocks of the server pass coming up between theirs (steps of
+// 6 x 10^7 elements, n = 1, took 441 us against 425, of 1.2 x 10^8, n = 2, 1235 against 1204), and for the rings, which
+// fill an SM's shared memory, no gain has been shown.
 __device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -1,8 +1,8 @@
-// The plain step kernels: the identity worker, the server pass for the streams the pipelined one
-// does not take and the stand-alone weight broadcast, grid-stride loops over a tile table; and what
-// the pipelined kernels share with them.
+// The plain step kernels: the identity worker, the stochastic operator in calls of few tiles, the server pass for the
+// streams the pipelined one does not take and the stand-alone weight broadcast, grid-stride loops over a tile table; and
+// what the pipelined kernels share with them.
 //
-// Thread/tile mapping (all kernels): a CTA of 256 threads owns a tile of up to
+// Thread/tile mapping (all kernels here): a CTA of 256 threads owns a tile of up to
 // 4096 consecutive padded elements as 4 CTA-wide rows of 1024; in row r thread t
 // owns the 4 consecutive elements starting at r*1024 + 4*t, so every global
 // access of fp32 state is one coalesced 128-bit access per thread, and one warp

@@ -224,7 +224,7 @@ __device__ __forceinline__ void fill_header(const WorkerParams& p, StreamHeader*
 // mille of a pair of 10^8 elements.
 // ---------------------------------------------------------------------------
 constexpr unsigned kListedPerRow = 4;                 // open elements of a row, at most, that are listed
-constexpr unsigned kListParts = 3;                    // warps a region of the list is dealt out to
+constexpr unsigned kListParts = 3;                    // warps a region is dealt out to (4 x 10^8 elements: 43.8 -> 41.7 us; few: 0.5 more)
 constexpr int kListBatch = 4;
 
 // BITS: code width, 2 (ternary) or 3 (five levels).
