@@ -499,10 +499,11 @@ def six_digits(v):
 
 def printed_line(line):
     """The line as it is printed; as many configurations from the end of the list as would make it
-    too long to be read back are left out."""
+    too long to be read back are left out, and counted."""
     line = six_digits(line)
     while len(json.dumps(line)) >= LINE_CHARS and line.get("configs"):
         line["configs"].pop()
+        line["configs_left_out"] = line.get("configs_left_out", 0) + 1
     return json.dumps(line)
 
 

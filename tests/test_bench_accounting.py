@@ -52,6 +52,12 @@ def test_two_full_passes_keep_a_record_each(monkeypatch):
     assert set(t) == {"absmax", "quantize"} and all(k["achieved_gbs"] > 0 for k in t.values())
 
 
+def test_configurations_the_printed_line_leaves_out_are_counted():
+    back = bench.json.loads(bench.printed_line({"value": 1.0, "configs": ["x" * 100] * 100}))
+    assert len(back["configs"]) + back["configs_left_out"] == 100 and back["configs_left_out"] > 0
+    assert "configs_left_out" not in bench.json.loads(bench.printed_line({"value": 1.0, "configs": ["x"]}))
+
+
 def test_the_printed_line_is_short_enough_to_be_read_back():
     rec = {"workload": "resnet18_qg_qx_k1", "n_workers": 8, "placement": "worker", "weight_decay": 5e-4,
            "weight_feedback": True, "ms_per_step": 0.0123456789, "step_frac": 0.123456}
